@@ -614,7 +614,7 @@ def time_forward(args, wl, L, bf16, stream, flush, torch, avtp, world, dev):
         torch.cuda.synchronize()
         ms = sorted(a.elapsed_time(b) for a, b in ev)
         out[key] = {"ms": reduce_max(sum(ms), world, dev) / K, "p50_us": round(ms[len(ms) // 2] * 1e3, 2),
-                    "launches": K * (7 if with_scores else 4)}  # k_prep, qtiles, transpose, forward (+ pack, mass, finalize)
+                    "launches": K * (5 if with_scores else 2)}  # k_prep, forward (+ pack, mass, finalize)
         del call
     return out, K
 
@@ -1107,7 +1107,7 @@ def run_timeline_forward(args):
     # the first CTA runs the last query tile of the last request: its key blocks
     cu = lay.cu_seqlens
     a, b = int(cu[-2]), int(cu[-1])
-    nblk = (b - 1) // 128 - a // 128 + 1
+    nblk = (b - a + 127) // 128
     n = min(nblk, 256)  # the timeline build keeps the first 256 blocks
     flush = L2Flush(dev)
     per_call = []
@@ -1131,8 +1131,8 @@ def run_timeline_forward(args):
     return {"config": args.config, "blocks": nblk, "blocks_stamped": n, "unit": "SM cycles per 128-key block (median)",
             "period": med(lambda t, j: t[j, S["p_handed"]] - t[j - 1, S["p_handed"]]),
             "softmax": {"wait_for_S": med(lambda t, j: t[j, S["s_ready"]] - t[j, S["top"]]),
-                        "load_mask_max_exchange": med(lambda t, j: t[j, S["exchanged"]] - t[j, S["s_ready"]]),
-                        "exponentials": med(lambda t, j: t[j, S["exp_done"]] - t[j, S["exchanged"]]),
+                        "first_half": med(lambda t, j: t[j, S["half_done"]] - t[j, S["s_ready"]]),
+                        "second_half": med(lambda t, j: t[j, S["exp_done"]] - t[j, S["half_done"]]),
                         "p_handover": med(lambda t, j: t[j, S["p_handed"]] - t[j, S["exp_done"]])},
             "mma_thread": {"S_waits_and_issue": med(lambda t, j: t[j, S["mma_s_issued"]] - t[j, S["mma_s_entry"]]),
                            "PV_waits": med(lambda t, j: t[j, S["mma_pv_ready"]] - t[j, S["mma_pv_entry"]]),

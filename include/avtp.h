@@ -231,8 +231,8 @@ AVTP_API avtp_status_t avtp_attn_forward(const avtp_layout_t* layout, const avtp
  * most 256; the rest of out is left untouched) key blocks. Available in the library's
  * timeline build (compiled with AVTP_TIMELINE); the default build returns
  * AVTP_ERR_UNSUPPORTED. out: host int64 [max_blocks][10]: per block j, from softmax warp 0
- * the loop top, S ready, the half maxima exchanged, the exponentials done and P handed
- * over, then from the MMA-issuing thread S_j's entry and issue and P_j V_j's entry,
+ * the loop top, S ready, P of the block's first 64 keys computed, P of the others computed
+ * and handed over, then from the MMA-issuing thread S_j's entry and issue and P_j V_j's entry,
  * operands ready and issue. Synchronises the device. */
 AVTP_API avtp_status_t avtp_forward_timeline(int64_t* out, int32_t max_blocks);
 

@@ -370,7 +370,7 @@ class ForwardCall:
         return self
 
 
-FORWARD_TIMELINE_SLOTS = ("top", "s_ready", "exchanged", "exp_done", "p_handed", "mma_s_entry", "mma_s_issued",
+FORWARD_TIMELINE_SLOTS = ("top", "s_ready", "half_done", "exp_done", "p_handed", "mma_s_entry", "mma_s_issued",
                           "mma_pv_entry", "mma_pv_ready", "mma_pv_issued")
 
 

@@ -167,12 +167,9 @@ WsPlan plan_workspace(const avtp_layout_t& L, const avtp_score_args_t* sa) {
   return p;
 }
 
-FwdWs plan_forward_workspace(const avtp_layout_t& L, const avtp_score_args_t& sa, size_t base_bytes) {
+FwdWs plan_forward_workspace(const avtp_layout_t& L, const avtp_score_args_t&, size_t base_bytes) {
   FwdWs f{};
   size_t off = align_up(base_bytes);
-  f.Tp = (L.n_tokens + 7) & ~static_cast<int64_t>(7);
-  f.vt = off;
-  off = align_up(off + static_cast<size_t>(sa.n_kv_heads) * sa.head_dim * static_cast<size_t>(f.Tp) * 2 + 16);
   f.qtile_cu = off;
   off = align_up(off + (static_cast<size_t>(L.n_requests) + 1) * 4);
   f.total = off;
@@ -312,6 +309,8 @@ avtp_status_t avtp_attn_forward(const avtp_layout_t* layout, const avtp_score_ar
   pa.zero_img_sums = img_sums;
   pa.build_text_tiles = scores != nullptr;
   if (pa.build_text_tiles) pa.attn = attn_plan(*layout, sa);
+  pa.qtile_cu = ws_at<int32_t>(workspace, f.qtile_cu);
+  pa.qtile_rows = forward_unit_rows(sa);
   if ((st = from_cuda(launch_prep(pa, workspace, p, s))) != AVTP_OK) return st;
   if ((st = from_cuda(launch_attn_forward(*layout, sa, *fwd_args, workspace, p, f, s))) != AVTP_OK) return st;
   if (scores == nullptr) return AVTP_OK;

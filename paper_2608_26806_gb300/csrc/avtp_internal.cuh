@@ -320,6 +320,9 @@ struct PrepArgs {
   int64_t* zero_img_sums;    // NULL: not zeroed
   int build_text_tiles;      // criterion B bookkeeping, sized by `attn`
   AttnPlan attn;
+  // The forward's units of qtile_rows query rows per request, as a prefix [R + 1]; NULL: none.
+  int32_t* qtile_cu;
+  int qtile_rows;
   // The image spans of the pruned batch (avtp_pruned_layout), from these budgets; NULL: none.
   const int32_t* pl_budgets;
   int32_t* pl_out_start;

@@ -5,8 +5,8 @@
 // Writes into the workspace: the status word, vis_cu (visual-token prefix over
 // all images), img_req (request of each image), and optionally the global
 // budgets B_r = floor(r_base * N_vis + 0.5) (paper §3.3.3 base keep ratio),
-// out_cu_seqlens, the text-query bookkeeping of the attention criterion, and the
-// image spans of the pruned batch (progressive pruning, paper §3.3.2).
+// out_cu_seqlens, the attention forward's unit prefix, the text-query bookkeeping of the
+// attention criterion, and the image spans of the pruned batch (progressive pruning, paper §3.3.2).
 #include "avtp_internal.cuh"
 
 namespace avtp {
@@ -164,6 +164,10 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
           a.out_cu_seqlens, s_warp);
     }
   }
+
+  if (s_err == 0 && a.qtile_cu != nullptr)
+    block_exclusive_scan<int32_t>(
+        R, [&](int r) { return (cu[r + 1] - cu[r] + a.qtile_rows - 1) / a.qtile_rows; }, a.qtile_cu, s_warp);
 
   if (s_err == 0 && a.build_text_tiles) {
     // Phase 4: text ordinals. Text ordinal of packed token t = t - (visual tokens before t).

@@ -221,3 +221,53 @@ def test_forward_strided_tensors():
     assert torch.all(o_big[:, Hq:] == 7.0) and torch.all(lse_big[:, T:] == 7.0)
     ref = O.score_text_attention(wl.layout, wl.q, wl.k, Hq, Hkv, wl.softmax_scale)
     assert_scores_close(c.scores.cpu().numpy(), ref, wl.layout.visual_mask())
+
+
+# ---------------------------------------------------------------- the softmax's reference, tile edges
+# A row's reference moves when a half block's sum of exponentials leaves its range: keys that
+# grow along the sequence move it again and again, in first and second halves of a block.
+@pytest.mark.parametrize("heads", [(4, 2, 64), (3, 1, 64), (8, 2, 128), (3, 3, 128)])
+@pytest.mark.parametrize("growth", [40.0, -40.0, 400.0])
+def test_forward_moving_reference(heads, growth):
+    Hq, Hkv, d = heads
+    wl = synth.make_custom([[("t", 3), ("i", 500), ("t", 27)], [("i", 64), ("t", 129)]], n_q_heads=Hq, n_kv_heads=Hkv,
+                           head_dim=d, hidden=64, seed=77, parts=("B", "V"))
+    T = wl.layout.n_tokens
+    rng = np.random.default_rng(5)
+    # logits that climb (or fall) by `growth` over 500 keys, in steps of their own size, the
+    # same for every query: q = 1 / d everywhere plus noise, k = ramp + noise
+    ramp = growth * (np.arange(T) // 37) * 37 / 500.0
+    scale = 1.0
+    q = (np.full((T, Hq, d), 1.0 / d) + 0.002 * rng.standard_normal((T, Hq, d))).astype(np.float32)
+    k = (ramp[:, None, None] + rng.standard_normal((T, Hkv, d))).astype(np.float32)
+    wl.tensors["q"] = synth.f32_to_bf16_bits(q.reshape(T, -1)).reshape(T, Hq, d)
+    wl.tensors["k"] = synth.f32_to_bf16_bits(k.reshape(T, -1)).reshape(T, Hkv, d)
+    L, qd, kd, vd = _dev(wl)
+    o, lse, _, _ = avtp.attn_forward(L, q=qd, k=kd, v=vd, softmax_scale=scale, scores=False)
+    torch.cuda.synchronize()
+    ref_o, ref_lse = O.attention_forward(wl.layout, wl.q, wl.k, wl.v, Hq, Hkv, scale)
+    ref_abs, _ = O.attention_forward(wl.layout, wl.q, wl.k, _abs_v(wl.v), Hq, Hkv, scale)
+    # fp32 logits of up to 440 (products of up to 7): their sum is off by at most d 2^-24 times
+    # sum |q k| = 128 * 2^-24 * 500 < 4e-3, which moves a probability by as much of itself
+    err = np.abs(o.cpu().numpy() - ref_o)
+    assert np.all(err <= (O_REL + (4e-3 if growth == 400.0 else 4e-4)) * ref_abs + 1e-5)
+    np.testing.assert_allclose(lse.cpu().numpy(), ref_lse, rtol=RTOL, atol=4e-3 if growth == 400.0 else 4e-4)
+
+
+@pytest.mark.parametrize("heads", [(4, 2, 64), (3, 1, 128)])
+@pytest.mark.parametrize("n", [1, 15, 16, 64, 65, 127, 128, 130, 255, 257])
+def test_forward_ignores_what_other_requests_hold(n, heads):
+    """A request's last tile reads rows of the next request: infinities and NaN there stay there."""
+    Hq, Hkv, d = heads
+    wl = synth.make_custom([[("i", 3), ("t", 2)], [("t", n)], [("t", 300)]], n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d,
+                           hidden=64, seed=100 + n, parts=("B", "V"))
+    ref_o, ref_lse = O.attention_forward(wl.layout, wl.q, wl.k, wl.v, Hq, Hkv, wl.softmax_scale)
+    ref_abs, _ = O.attention_forward(wl.layout, wl.q, wl.k, _abs_v(wl.v), Hq, Hkv, wl.softmax_scale)
+    L, q, k, v = _dev(wl)
+    for t, x in ((q, float("nan")), (k, float("inf")), (v, float("nan"))):
+        t[:5], t[5 + n:] = x, x
+    o, lse, _, _ = avtp.attn_forward(L, q=q, k=k, v=v, softmax_scale=wl.softmax_scale, scores=False)
+    torch.cuda.synchronize()
+    mine = slice(5, 5 + n)
+    _check_o(o.cpu().numpy()[mine], ref_o[mine], ref_abs[mine])
+    np.testing.assert_allclose(lse.cpu().numpy()[:, mine], ref_lse[:, mine], rtol=RTOL, atol=ATOL)
