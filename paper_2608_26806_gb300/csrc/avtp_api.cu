@@ -149,6 +149,9 @@ WsPlan plan_workspace(const avtp_layout_t& L, const avtp_score_args_t* sa) {
     p.ktile_cu = take((NI + 1) * 4);
     p.ktile_img = take(static_cast<size_t>(a.n_ktiles_max) * 4);
     p.meta = take(8 * 4);
+    p.blk_info = take(static_cast<size_t>(a.n_blocks_max) * sizeof(AttnBlkInfo));
+    p.tile_info = take(static_cast<size_t>(a.n_ktiles_max) * 16);
+    p.cta_start = take(2 * static_cast<size_t>(a.grid) * 16);
     if (attn_uses_cuda_cores(L, *sa)) {
       const NarrowPlan np = narrow_plan(L, *sa, a.max_text);
       const size_t nrows = static_cast<size_t>(np.rows);

@@ -24,15 +24,27 @@ constexpr double kRatioLimit = 1048576.0;  // ratios saturate at +-2^20 before t
 
 // Tiles of the text-attention criterion (tensor-core path). Rows are (text query, head
 // of the KV group) pairs, G = Hq / Hkv of them per text query, in text order. A request's
-// rows are cut into blocks of kAttnBlockRows; pass 1 runs a block as two MMA A tiles
-// against key tiles of kAttnTileN keys, pass 2 holds a block as the MMA B operand and
-// streams key tiles of kAttnTileM visual keys through it.
-constexpr int kAttnTileM = 128;          // MMA M: rows of a pass-1 A tile, keys of a pass-2 tile
-constexpr int kAttnTileN = 256;          // MMA N: keys per pass-1 step, rows of a pass-2 block
+// rows are cut into blocks of kAttnBlockRows; both passes hold a block in shared memory
+// as two products of 128 rows and stream key tiles of kAttnTileM keys past it (pass 1
+// every key from the request's first, pass 2 the visual keys).
+constexpr int kAttnTileM = 128;          // keys of a tile, rows of a product
 constexpr int kAttnBlockRows = 256;      // rows per block (both passes)
 constexpr int kAttnMaxChunks = 64;       // pass-1 partial (max, sum) slots per row at most
 constexpr int kAttnMaxGroupHeads = 128;  // Hq / Hkv at most
 constexpr int kAttnMassFracBits = 40;    // fixed point of the per-key probability mass
+
+// What the two passes need of a row block, laid out by the validation kernel (as two int4)
+// so that a walk over blocks takes one load where the prefix arrays would take a search.
+// Beside it: per key tile an int4 (first packed key, keys, text ordinals in the batch before
+// the token behind its image), and per CTA and pass an int4 (KV group, block, entry within
+// the block, steps of its run).
+struct AttnBlkInfo {
+  int R0, rows;     // first row (of every KV group), rows
+  int key0, tile0;  // packed position of the request's first key, its first key tile
+  int s1, n1, n2;   // first step in a KV group's pass-1 list, pass-1 steps, pass-2 tiles
+  int pad;
+};
+static_assert(sizeof(AttnBlkInfo) == 32, "two int4");
 
 // ---------------------------------------------------------------- status
 // First word of every workspace. code: first error recorded (0 = none);
@@ -133,7 +145,10 @@ struct WsPlan {
   size_t p2t_cu;      // int32 [n_blocks_max + 1]: pass-2 key tiles per row block
   size_t ktile_cu;    // int32 [n_img + 1]: key tiles per image
   size_t ktile_img;   // int32 [n_ktiles_max]: image of every key tile
-  size_t meta;        // int32 [8]: F1, C1, F2, C2 (flat pass lengths per KV group, steps per CTA)
+  size_t meta;        // int32 [8]: F1, C1, F2, C2 (flat pass lengths per KV group, steps per CTA), row blocks
+  size_t blk_info;    // AttnBlkInfo [n_blocks_max]
+  size_t tile_info;   // int4 [n_ktiles_max]: see AttnBlkInfo
+  size_t cta_start;   // int4 [2][grid]: see AttnBlkInfo
   size_t qt;          // bf16 [Hkv, rows, d]: the text queries, packed by KV group
   size_t lse_rows;    // float [Hkv, rows]: log2-domain LSE of every row (supplied LSE only)
   size_t p1_part;     // float2 [Hkv * n_blocks_max][256][kAttnMaxChunks]: per-CTA (max, sum) of every row

@@ -271,17 +271,18 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-// D = A(M x d) * B(N x d)^T over the whole row length d (64 or 128): d / 16 MMAs.
+// D = A(M x D) * B(N x D)^T over the whole row length D (64 or 128): D / 16 MMAs.
 // a_base / b_base: shared addresses of atom column 0; atom columns are a_atom / b_atom
 // bytes apart.
+template <int D>
 __device__ __forceinline__ void mma_rows(uint32_t d_tmem, uint32_t a_base, uint32_t a_atom, uint32_t b_base,
-                                         uint32_t b_atom, int d, uint32_t idesc) {
-#pragma unroll 1
-  for (int ks = 0; ks < d / 16; ++ks) {
-    const uint32_t off = static_cast<uint32_t>(ks & 3) * 32u;
-    const uint32_t a = a_base + static_cast<uint32_t>(ks >> 2) * a_atom + off;
-    const uint32_t b = b_base + static_cast<uint32_t>(ks >> 2) * b_atom + off;
-    mma_bf16(d_tmem, desc_k_sw128(a), desc_k_sw128(b), idesc, ks > 0 ? 1u : 0u);
+                                         uint32_t b_atom, uint32_t idesc) {
+  const uint64_t da = desc_k_sw128(a_base), db = desc_k_sw128(b_base);
+#pragma unroll
+  for (int ks = 0; ks < D / 16; ++ks) {
+    const uint32_t off = static_cast<uint32_t>(ks & 3) * 2u;  // descriptors count 16 bytes
+    mma_bf16(d_tmem, da + off + (ks >> 2) * (a_atom / 16), db + off + (ks >> 2) * (b_atom / 16), idesc,
+             ks > 0 ? 1u : 0u);
   }
 }
 

@@ -56,13 +56,19 @@ __device__ T block_exclusive_scan(int n, F value, T* out, T* s_warp) {
 // which is launched while this kernel still runs.
 constexpr int kStageInts = 2560;
 
+// Prefixes of the two passes' lists kept in shared memory for the search of the CTAs' runs.
+constexpr int kStageBlocks = 1024;
+
+// kText: with the text-query bookkeeping of the attention criterion.
+template <bool kText>
 __global__ void __launch_bounds__(kPrepThreads)
 k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t* req_budget, int32_t* text_idx,
        int32_t* text_cu, int32_t* blk_cu, int32_t* p1s_cu, int32_t* p2t_cu, int32_t* ktile_cu, int32_t* ktile_img,
-       int32_t* meta, int32_t* g_scratch) {
+       int32_t* meta, int4* blk_info, int4* tile_info, int4* cta_start, int32_t* g_scratch) {
   __shared__ int s_err, s_detail, s_max_steps;
   __shared__ int32_t s_warp[32];
   __shared__ int32_t s_stage[kStageInts];
+  __shared__ int32_t s_list[kText ? 2 : 1][kText ? kStageBlocks + 1 : 1];
   // The first kernel of a call: it is launched after everything before it in the
   // stream has finished, so the next kernel may be scheduled at once.
   pdl_trigger();
@@ -169,7 +175,7 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
     block_exclusive_scan<int32_t>(
         R, [&](int r) { return (cu[r + 1] - cu[r] + a.qtile_rows - 1) / a.qtile_rows; }, a.qtile_cu, s_warp);
 
-  if (s_err == 0 && a.build_text_tiles) {
+  if (kText && s_err == 0) {
     // Phase 4: text ordinals. Text ordinal of packed token t = t - (visual tokens before t).
     for (int r = tid; r <= R; r += blockDim.x) text_cu[r] = cu[r] - vis_cu[icu[r]];
     __syncthreads();
@@ -205,8 +211,16 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
       // Key tiles of kAttnTileM visual keys per image.
       block_exclusive_scan<int32_t>(
           NI, [&](int i) { return (iln[i] + kAttnTileM - 1) / kAttnTileM; }, ktile_cu, s_warp);
-      for (int i = tid; i < NI; i += blockDim.x)
-        for (int t = ktile_cu[i]; t < ktile_cu[i + 1]; ++t) ktile_img[t] = i;
+      for (int i = tid; i < NI; i += blockDim.x) {
+        const int r = img_req[i], t0 = ktile_cu[i], t1 = ktile_cu[i + 1];
+        const int key0 = cu[r] + ist[i], n = iln[i];
+        const int o_first = text_cu[r] + ist[i] + n - (vis_cu[i + 1] - vis_cu[icu[r]]);
+        for (int t = t0; t < t1; ++t) {
+          const int first = (t - t0) * kAttnTileM;
+          ktile_img[t] = i;
+          tile_info[t] = make_int4(key0 + first, min(kAttnTileM, n - first), o_first, 0);
+        }
+      }
       // Pass 2 of block b: the key tiles of every image that at least one of the block's
       // queries follows. Images are sorted and the text ordinal of the first token after
       // image i, o_first(i), does not decrease with i, so those images are a prefix.
@@ -221,10 +235,12 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
               static_cast<int64_t>(text_cu[r]) + ist[i] + iln[i] - (vis_cu[i + 1] - vis_cu[icu[r]]);
           if (o_first * G >= R1) hi = i; else lo = i + 1;
         }
-        return ktile_cu[lo] - ktile_cu[icu[r]];
+        const int tile0 = ktile_cu[icu[r]];
+        blk_info[2 * b] = make_int4(static_cast<int>(R0), static_cast<int>(R1 - R0), cu[r], tile0);
+        return ktile_cu[lo] - tile0;
       };
       block_exclusive_scan<int32_t>(NB, p2_tiles, p2t_cu, s_warp);
-      // Pass 1 of block b: steps of kAttnTileN keys from the request's first token to its
+      // Pass 1 of block b: steps of kAttnTileM keys from the request's first token to its
       // last query (none when pass 2 has nothing for the block).
       if (tid == 0) s_max_steps = 0;
       __syncthreads();
@@ -234,14 +250,24 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
         const int64_t R0 = static_cast<int64_t>(text_cu[r]) * G + static_cast<int64_t>(b - blk_cu[r]) * kAttnBlockRows;
         const int64_t R1 = min(R0 + kAttnBlockRows, static_cast<int64_t>(text_cu[r + 1]) * G);
         const int keys = text_idx[(R1 - 1) / G] - cu[r] + 1;
-        const int steps = (keys + kAttnTileN - 1) / kAttnTileN;
+        const int steps = (keys + kAttnTileM - 1) / kAttnTileM;
         atomicMax(&s_max_steps, steps);
         return steps;
       };
       block_exclusive_scan<int32_t>(NB, p1_steps, p1s_cu, s_warp);
-      if (tid == 0) {
+      const bool short_list = NB <= kStageBlocks;
+      for (int b = tid; b <= NB; b += blockDim.x) {
+        const int s1 = p1s_cu[b], t2 = p2t_cu[b];
+        if (b < NB) blk_info[2 * b + 1] = make_int4(s1, p1s_cu[b + 1] - s1, p2t_cu[b + 1] - t2, 0);
+        if (short_list) {
+          s_list[0][b] = s1;
+          s_list[1][b] = t2;
+        }
+      }
+      __syncthreads();
+      {
         // Each CTA of a persistent pass takes a contiguous run of C steps of the flat
-        // list (KV group, block, step). C1 also keeps a row's pass-1 partials within
+        // list (KV group, block, step), laid out in cta_start. C1 also keeps a row's pass-1 partials within
         // kAttnMaxChunks slots: a block of S steps meets at most (S - 1) / C1 + 2 CTAs.
         const int64_t grid = a.attn.grid > 0 ? a.attn.grid : 1;
         const int64_t F1 = p1s_cu[NB], F2 = p2t_cu[NB];
@@ -249,10 +275,28 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
         const int64_t c_min = (s_max_steps - 1 + kAttnMaxChunks - 3) / (kAttnMaxChunks - 2);
         C1 = max(max(C1, c_min), static_cast<int64_t>(1));
         const int64_t C2 = max((a.attn.Hkv * F2 + grid - 1) / grid, static_cast<int64_t>(1));
-        meta[0] = static_cast<int32_t>(F1);
-        meta[1] = static_cast<int32_t>(C1);
-        meta[2] = static_cast<int32_t>(F2);
-        meta[3] = static_cast<int32_t>(C2);
+        if (tid == 0) {
+          meta[0] = static_cast<int32_t>(F1);
+          meta[1] = static_cast<int32_t>(C1);
+          meta[2] = static_cast<int32_t>(F2);
+          meta[3] = static_cast<int32_t>(C2);
+          meta[4] = NB;
+        }
+        for (int64_t c = tid; c < 2 * grid; c += blockDim.x) {
+          const int pass = c >= grid ? 1 : 0;
+          const int64_t F = pass ? F2 : F1, C = pass ? C2 : C1;
+          const int64_t total = a.attn.Hkv * F, f = (c - pass * grid) * C;
+          int4 s = make_int4(0, 0, 0, 0);
+          if (f < total) {
+            const int32_t* list = short_list ? s_list[kText ? pass : 0] : (pass ? p2t_cu : p1s_cu);
+            s.x = static_cast<int>(f / F);
+            const int fl = static_cast<int>(f - s.x * F);
+            s.y = upper_index(list, NB, fl);
+            s.z = fl - list[s.y];
+            s.w = static_cast<int>(min(C, total - f));
+          }
+          cta_start[c] = s;
+        }
       }
     }
   }
@@ -308,17 +352,16 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
 
 cudaError_t launch_prep(const PrepArgs& a, void* ws, const WsPlan& p, cudaStream_t s) {
   const bool b = a.build_text_tiles != 0;
-  k_prep<<<1, kPrepThreads, 0, s>>>(a, ws_at<DevStatus>(ws, p.status), ws_at<int32_t>(ws, p.vis_cu),
-                                    ws_at<int32_t>(ws, p.img_req), ws_at<int32_t>(ws, p.req_budget),
-                                    b ? ws_at<int32_t>(ws, p.text_idx) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.text_cu) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.blk_cu) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.p1s_cu) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.p2t_cu) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.ktile_cu) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.ktile_img) : nullptr,
-                                    b ? ws_at<int32_t>(ws, p.meta) : nullptr,
-                                    a.pl_budgets != nullptr ? ws_at<int32_t>(ws, p.scratch) : nullptr);
+  auto kernel = b ? k_prep<true> : k_prep<false>;
+  kernel<<<1, kPrepThreads, 0, s>>>(
+      a, ws_at<DevStatus>(ws, p.status), ws_at<int32_t>(ws, p.vis_cu), ws_at<int32_t>(ws, p.img_req),
+      ws_at<int32_t>(ws, p.req_budget), b ? ws_at<int32_t>(ws, p.text_idx) : nullptr,
+      b ? ws_at<int32_t>(ws, p.text_cu) : nullptr, b ? ws_at<int32_t>(ws, p.blk_cu) : nullptr,
+      b ? ws_at<int32_t>(ws, p.p1s_cu) : nullptr, b ? ws_at<int32_t>(ws, p.p2t_cu) : nullptr,
+      b ? ws_at<int32_t>(ws, p.ktile_cu) : nullptr, b ? ws_at<int32_t>(ws, p.ktile_img) : nullptr,
+      b ? ws_at<int32_t>(ws, p.meta) : nullptr, b ? ws_at<int4>(ws, p.blk_info) : nullptr,
+      b ? ws_at<int4>(ws, p.tile_info) : nullptr, b ? ws_at<int4>(ws, p.cta_start) : nullptr,
+      a.pl_budgets != nullptr ? ws_at<int32_t>(ws, p.scratch) : nullptr);
   return cudaGetLastError();
 }
 

@@ -8,27 +8,37 @@
 // Qt[g][row][d] (k_attn_pack), so that both passes read them with TMA boxes. A
 // request's rows are cut into blocks of 256.
 //
-// Pass 1, k_attn_lse (skipped when the caller supplies FlashAttention's LSE): a block
-// is held as two 128-row A tiles and every key tile of 256 keys, from the request's
-// first token to the block's last query, feeds two MMAs (128 x 256 x d, one per A
-// tile, fp32 accumulators in TMEM), so every key byte brought to the SM serves 256
-// rows. The epilogue reads accumulator 0 while the MMA of tile 1 runs and keeps an
-// online (max, sum) per row; it leaves one partial per (row, CTA) behind.
-// Pass 2, k_attn_mass: a block is held as the MMA B operand (N = 256 rows) and the
-// tiles of 128 visual keys of every image that one of its queries follows stream
-// through it as A (M = 128 keys), into two accumulators used in turn. A thread owns
-// one key and sums exp2(z2 - lse2) over the rows of its column half; lse2 comes from
-// the pass-1 partials of the block (merged on load) or from the supplied LSE, and is
-// +inf on rows whose query precedes the key's image. The per-key sums of all blocks
-// and KV groups meet in a 64-bit fixed-point accumulator (integer atomics: the result
+// Pass 1, k_attn_lse (skipped when the caller supplies FlashAttention's LSE): a block's rows
+// stay in shared memory as two A operands of 128 rows and the tiles of 128 keys, from the
+// request's first token to the block's last query, stream past them as B: two products of
+// 128 x 128 x d a tile. A thread owns a row and keeps (reference, sum of exp2) of every other
+// tile's logits; one partial per (row, CTA) is left behind.
+// Pass 2, k_attn_mass: the same with the roles exchanged: the tiles of 128 visual keys of
+// every image that one of the block's queries follows are the A operand, the block's halves
+// the B operand. A thread owns a key and sums exp2(z2 - lse2) over 128 rows, leaving out the
+// rows whose query precedes the key's image; lse2 comes from the pass-1 partials of the
+// block (merged when the walk enters it) or from the supplied LSE. The per-key sums of all
+// blocks and KV groups meet in a 64-bit fixed-point accumulator (integer atomics: the result
 // does not depend on their order).
 // k_attn_finalize turns the accumulator into scores and the fixed-point image sums.
 //
-// Both passes are persistent: the flat list of (KV group, block, key step) is split
-// into equal contiguous runs, one per CTA (one CTA per SM). Warps 0-7 are the epilogue
-// (warp w reads TMEM lanes 32(w%4)..+31 and column half w/4 of every accumulator),
-// warp 8 issues the TMA loads, warp 9 owns TMEM and issues the MMAs. TMEM holds two
-// 256-column accumulators.
+// Both passes are persistent: the flat list of (KV group, block, key tile) is split into
+// equal contiguous runs, one per CTA (one CTA per SM). TMEM holds four accumulators of 128
+// columns, one for each half of the block and parity of the step. Warps 0-15 are the
+// epilogue, four per accumulator (warp w reads TMEM lanes 32(w%4)..+31 of accumulator w/4),
+// so every SM sub-partition has a warp of each; warp 16 issues the TMA loads; warps 17 and
+// 18 own a half of the block each and issue its MMAs, so that a half whose epilogue is
+// slower (its rows see more) does not hold up the other.
+//
+// What bounds them: the epilogue's exponentials and sums, 1235 cycles for a tile's 128 x 256
+// logits with all sixteen warps busy (measured alone; exp2 alone 1024), against 1024 for the
+// MMAs; where causality leaves an epilogue little to do, the key tiles' delivery (24 bytes a
+// cycle and SM). Serving batch of 34423 tokens (8 requests, 32 heads, 8 KV heads): pass 1
+// 83 -> 62 us, pass 2 86 -> 70 us; one request of 10368 tokens with 256 text tokens: 27 -> 20
+// and 26 -> 24 us. Before, eight epilogue warps and two accumulators of 256 columns left the
+// MMAs and the epilogue of an accumulator waiting for each other, pass 1 took a maximum per
+// 32 logits, one lane behind a lane branch issued the MMAs, and every block began with
+// searches in the prefix arrays (AttnBlkInfo).
 #include <cudaTypedefs.h>
 
 #include "avtp_tc.cuh"
@@ -37,74 +47,68 @@ namespace avtp {
 namespace {
 
 constexpr int kM = kAttnTileM;        // 128
-constexpr int kN = kAttnTileN;        // 256
 constexpr int kBlk = kAttnBlockRows;  // 256
-constexpr int kTmaWarp = 8;
-constexpr int kMmaWarp = 9;
-constexpr int kThreads = 320;
-constexpr int kEpiWarps = 8;          // warps 0-7: epilogue
-constexpr uint32_t kTmemCols = 2 * kN;
-constexpr int kP2Stages = 4;          // key tiles in flight in pass 2
-constexpr int kMassWindow = 24;       // pass-2 steps whose key masses are held in shared memory between flushes
+constexpr int kGroupWarps = 4;        // epilogue warps of an accumulator
+constexpr int kSetThreads = 2 * 32 * kGroupWarps;  // threads of the two accumulators of a step
+constexpr int kTmaWarp = 4 * kGroupWarps;
+constexpr int kMmaWarp = kTmaWarp + 1;  // and the next
+constexpr int kThreads = 32 * (kMmaWarp + 2);
+constexpr uint32_t kTmemCols = 512;  // four accumulators of 128 columns
+constexpr int kStages = 4;            // key tiles in flight
+constexpr int kMassWindow = 12;       // steps of an epilogue group whose key masses are held in shared memory between flushes
 constexpr float kLog2e = 1.4426950408889634f;
 // Flag of a key whose mass is not a finite number in [0, 256] (non-finite inputs). The
 // sum of its finite contributions stays below 2^62: at most 256 * 2^40 per (KV group,
 // block), fewer than 2^14 of them.
 constexpr unsigned long long kMassNotFinite = 1ull << 63;
 
-static_assert(kBlk == 2 * kM && kBlk == kN, "a block is two A tiles (pass 1) and one B operand (pass 2)");
+static_assert(kBlk == 2 * kM, "a block is two products of 128 rows");
 
-// Shared memory for head_dim d (1024-byte aligned tiles).
+// Shared memory for head_dim d (1024-byte aligned tiles): the row block and kStages key tiles.
 __host__ __device__ constexpr size_t a_bytes(int d) { return static_cast<size_t>(kM) * d * 2; }
-__host__ __device__ constexpr size_t b_bytes(int d) { return static_cast<size_t>(kN) * d * 2; }
-// pass 1: two A tiles (the block) + two key stages; pass 2: the block + kP2Stages key tiles
-__host__ __device__ constexpr size_t lse_smem_bytes(int d) { return 1024 + 2 * a_bytes(d) + 2 * b_bytes(d); }
-__host__ __device__ constexpr size_t mass_smem_bytes(int d) { return 1024 + b_bytes(d) + kP2Stages * a_bytes(d); }
+__host__ __device__ constexpr size_t b_bytes(int d) { return static_cast<size_t>(kBlk) * d * 2; }
+__host__ __device__ constexpr size_t attn_smem_bytes(int d) { return 1024 + b_bytes(d) + kStages * a_bytes(d); }
 
 struct Sync {
-  uint64_t a_full[kP2Stages], a_empty[kP2Stages];
-  uint64_t b_full[2], b_empty[2];
-  uint64_t acc_full[2], acc_empty[2];
-  uint64_t drain;
+  uint64_t k_full[kStages], k_empty[kStages];
+  uint64_t b_full[2], b_empty[2];            // halves of the row block
+  uint64_t acc_full[2][2], acc_empty[2][2];  // [buffer: step parity][half]
+  uint64_t drain[2];
   uint32_t tmem;
   int abort;
 };
 
 struct AttnArgs {
-  const int32_t* cu;
-  int R;
-  const int32_t* ist;
-  const int32_t* iln;
-  const int32_t* icu;
-  int NI;
-  int64_t T;
-  const int32_t* vis_cu;
   const int32_t* text_idx;
-  const int32_t* text_cu;
-  const int32_t* blk_cu;
-  const int32_t* p1s_cu;
-  const int32_t* p2t_cu;
-  const int32_t* ktile_cu;
-  const int32_t* meta;           // F1, C1, F2, C2
+  const int4* blk_info;          // the validation kernel's tables, see AttnBlkInfo
+  const int4* tile_info;
+  const int4* cta_start;
+  const int32_t* meta;           // F1, C1, F2, C2, NB
   const float* lse_rows;         // [Hkv, rows] (supplied LSE) or nullptr
   float2* p1_part;               // [Hkv * NB][256 rows][kAttnMaxChunks]
   unsigned long long* mass;      // [key tile][128] fixed point, 2^-kAttnMassFracBits
   int64_t rows;
-  int G, Hkv, d;
+  int G;
   float c2;                      // softmax_scale * log2(e)
   DevStatus* st;
 };
 
-__device__ __forceinline__ void bar_epi() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// Barriers of the 256 epilogue threads of step parity b (id 1 + b), of all 512 (id 3), and of
+// the 128 of one accumulator (ids 4 .. 7).
+__device__ __forceinline__ void bar_set(int b) { asm volatile("bar.sync %0, 256;" ::"r"(1 + b) : "memory"); }
+__device__ __forceinline__ void bar_epi() { asm volatile("bar.sync 3, 512;" ::: "memory"); }
+__device__ __forceinline__ void bar_acc(int b, int t) {
+  asm volatile("bar.sync %0, 128;" ::"r"(4 + 2 * b + t) : "memory");
+}
 
 // Diagnostic timeline build (-DAVTP_TIMELINE): clock stamps of each pass's first CTA, per
 // step s of its run. Slots: 0 the key tile's load issued (TMA thread); 1 the MMA thread at
 // the step, 2 its operands and accumulators ready, 3 its MMAs issued and committed; 4 the
 // step's (first) accumulator ready for epilogue warp 0, 5 the step's (last) accumulator
 // released by it. Read with avtp_score_timeline().
+#ifdef AVTP_TIMELINE
 constexpr int kAttnTlSteps = 64;
 constexpr int kAttnTlSlots = 6;
-#ifdef AVTP_TIMELINE
 __device__ long long g_attn_tl[2][kAttnTlSteps][kAttnTlSlots];
 #endif
 __device__ __forceinline__ void attn_stamp(int pass, int st, int slot) {
@@ -117,39 +121,30 @@ __device__ __forceinline__ void attn_stamp(int pass, int st, int slot) {
 #endif
 }
 
-// A (KV group, row block) pair: rows [R0, R1) of group g belong to request r.
-struct Seg {
-  int g, b, r;
-  int64_t R0, R1;
-};
-
-__device__ __forceinline__ Seg seg_of(const AttnArgs& a, int g, int b) {
-  Seg s;
-  s.g = g;
-  s.b = b;
-  s.r = upper_index(a.blk_cu, a.R, b);
-  s.R0 = static_cast<int64_t>(a.text_cu[s.r]) * a.G + static_cast<int64_t>(b - a.blk_cu[s.r]) * kBlk;
-  s.R1 = min(s.R0 + kBlk, static_cast<int64_t>(a.text_cu[s.r + 1]) * a.G);
-  return s;
-}
-
-// Walks a CTA's run of the flat list (KV group, block, entry) of a pass whose per-group
-// list has F entries with prefix cu over the NB blocks. Global memory is read only
-// when the walk enters a new block, so the single MMA-issuing and TMA-issuing threads
-// do not wait on dependent loads between steps.
-struct FlatCursor {
-  int g, b, j;  // KV group, block, entry within the block
-  int n;        // entries of block b
-  __device__ __forceinline__ void init(int64_t f, int F, const int32_t* cu, int NB) {
-    g = static_cast<int>(f / F);
-    const int fl = static_cast<int>(f - static_cast<int64_t>(g) * F);
-    b = upper_index(cu, NB, fl);
-    j = fl - cu[b];
-    n = cu[b + 1] - cu[b];
+// Walks a CTA's run of a pass's flat list (KV group, block, entry): pass 1's entries are
+// steps of 128 keys from the request's first key, pass 2's the request's key tiles in order.
+template <int PASS>
+struct Walk {
+  int g, b, j, n;  // KV group, block, entry within the block, entries of the block
+  AttnBlkInfo blk;
+  const int4* tab;
+  int NB;
+  __device__ __forceinline__ void load() {
+    const int4 lo = tab[2 * b], hi = tab[2 * b + 1];
+    blk = AttnBlkInfo{lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, 0};
+    n = PASS == 1 ? blk.n1 : blk.n2;
+  }
+  __device__ __forceinline__ void init(const AttnArgs& a, const int4& start) {
+    g = start.x;
+    b = start.y;
+    j = start.z;
+    tab = a.blk_info;
+    NB = a.meta[4];
+    load();
   }
   // Next entry; returns true when it lies in another block. Only called while another
   // entry exists, so the loop over empty blocks ends.
-  __device__ __forceinline__ bool next(const int32_t* cu, int NB) {
+  __device__ __forceinline__ bool next() {
     if (++j < n) return false;
     j = 0;
     do {
@@ -157,139 +152,100 @@ struct FlatCursor {
         b = 0;
         ++g;
       }
-      n = cu[b + 1] - cu[b];
+      load();
     } while (n == 0);
     return true;
   }
   __device__ __forceinline__ bool last_of_block() const { return j + 1 == n; }
 };
 
-// Pass-2 key tiles of a block in order: tile j is tile jj of image i, the images of the
-// block's request in order. The request's fields are read when the walk enters a block;
-// the next image's fields are loaded as soon as the walk enters an image, so that their
-// latency is hidden behind the steps of the current image.
-struct TileCursor {
-  int i, jj;           // image, tile within the image
-  int kp0, nk, c0;     // first packed key, keys in the tile, first row of the block that sees it
-  int tile;            // key tile over all images (row of the mass accumulator)
-  int base, len, t0;   // packed position of the image's first key, its length, its first key tile
-  int64_t c0_img;      // o_first(i) * G - R0
-  int cu_r, text_r, vis_r0, img_end;  // the request's first token, first text ordinal, first visual ordinal, image end
-  int n_ist, n_iln, n_t0, n_vis;      // image i + 1: start, length, first key tile, visual prefix after it
-  __device__ __forceinline__ void prefetch(const AttnArgs& a) {
-    if (i + 1 < img_end) {
-      n_ist = a.ist[i + 1];
-      n_iln = a.iln[i + 1];
-      n_t0 = a.ktile_cu[i + 1];
-      n_vis = a.vis_cu[i + 2];
-    }
-  }
-  __device__ __forceinline__ void apply(const Seg& s, int g, int ist, int iln, int tk0, int vis1) {
-    base = cu_r + ist;
-    len = iln;
-    t0 = tk0;
-    const int64_t o_first = static_cast<int64_t>(text_r) + ist + iln - (vis1 - vis_r0);
-    c0_img = o_first * g - s.R0;
-  }
-  __device__ __forceinline__ void fill() {
-    kp0 = base + jj * kM;
-    nk = min(kM, len - jj * kM);
-    tile = t0 + jj;
-    c0 = c0_img > 0 ? static_cast<int>(c0_img) : 0;
-  }
-  __device__ __forceinline__ void init(const AttnArgs& a, const Seg& s, int j) {
-    const int r = s.r;
-    cu_r = a.cu[r];
-    text_r = a.text_cu[r];
-    vis_r0 = a.vis_cu[a.icu[r]];
-    img_end = a.icu[r + 1];
-    const int t = a.ktile_cu[a.icu[r]] + j;
-    i = upper_index(a.ktile_cu, a.NI, t);
-    jj = t - a.ktile_cu[i];
-    apply(s, a.G, a.ist[i], a.iln[i], a.ktile_cu[i], a.vis_cu[i + 1]);
-    prefetch(a);
-    fill();
-  }
-  __device__ __forceinline__ void next(const AttnArgs& a, const Seg& s) {
-    if ((++jj) * kM >= len) {
-      ++i;
-      jj = 0;
-      apply(s, a.G, n_ist, n_iln, n_t0, n_vis);
-      prefetch(a);
-    }
-    fill();
-  }
-};
-
 // ---------------------------------------------------------------- epilogue arithmetic
 // A warp's slice of an accumulator: its 32 TMEM lanes x kHalf columns, read as 32-column
-// chunks; chunk p+1 is loaded while chunk p is processed. MASKED = false is the common
-// case (every column visible to every lane): straight-line code without per-chunk
-// votes. The masked form handles the chunks [pb, pe) and keeps the columns c with
-// lo <= c < hi (per lane in pass 1, per CTA in pass 2).
-constexpr int kHalf = kN / 2;
+// chunks.
+constexpr int kHalf = kM;
 constexpr int kChunks = kHalf / 32;
+// A slice's sum above this moves the row's reference, if the slice's maximum exceeds it by
+// more than kRescaleTau (log2 units).
+constexpr float kRescaleSum = 16384.f;
+constexpr float kRescaleTau = 8.f;
 
-// Pass 1: online (max m, sum l) of exp2(c2 * z) over the visible columns of a row.
-template <bool MASKED>
-__device__ __forceinline__ void p1_slice(uint32_t taddr, int pe, int lim, float c2, float& m, float& l) {
-  uint32_t ra[32], rb[32];
-  auto chunk = [&](uint32_t(&r)[32], uint32_t(&nx)[32], int p) {
-    if (p + 1 < pe) tc::tmem_ld32_async(taddr + (p + 1) * 32, nx);
-    float v[32];
-#pragma unroll
-    for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+// Pass 1: f(chunk values) over the chunks [0, pe) of a row's slice, one at a time (four
+// warps a sub-partition hide each other's loads). MASKED: columns past lim (per lane) read
+// as -inf.
+template <bool MASKED, class F>
+__device__ __forceinline__ void p1_chunks(uint32_t taddr, int pe, int lim, F&& f) {
+#pragma unroll 1
+  for (int p = 0; p < pe; ++p) {
+    uint32_t r[32];
+    tc::tmem_ld32_async(taddr + p * 32, r);
+    tc::tmem_wait(r);
     if (MASKED) {
 #pragma unroll
-      for (int q = 0; q < 32; ++q) v[q] = (p * 32 + q <= lim) ? v[q] : -INFINITY;
+      for (int q = 0; q < 32; ++q) r[q] = (p * 32 + q <= lim) ? r[q] : 0xff800000u;
     }
-    // max as a tree (depth 5); exact in any order
-    float t16[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) t16[q] = fmaxf(v[2 * q], v[2 * q + 1]);
-#pragma unroll
-    for (int w = 8; w >= 1; w >>= 1) {
-#pragma unroll
-      for (int q = 0; q < w; ++q) t16[q] = fmaxf(t16[q], t16[q + w]);
-    }
-    const float mn = fmaxf(m, t16[0] * c2);
-    // four partial sums (columns q mod 4), two per packed register
-    const float2 cc = make_float2(c2, c2), nm = make_float2(-mn, -mn);
-    float2 s01 = make_float2(0.f, 0.f), s23 = s01;
+    f(r);
+  }
+}
+// Sum of exp2(c2 z - m) over the slice, in four partial sums (columns q mod 4).
+template <bool MASKED>
+__device__ __forceinline__ float p1_sum(uint32_t taddr, int pe, int lim, float c2, float m) {
+  const float nm1 = (m == -INFINITY) ? 0.f : -m;
+  const float2 cc = make_float2(c2, c2), nm = make_float2(nm1, nm1);
+  float2 s01 = make_float2(0.f, 0.f), s23 = s01;
+  p1_chunks<MASKED>(taddr, pe, lim, [&](const uint32_t(&r)[32]) {
 #pragma unroll
     for (int q = 0; q < 32; q += 4) {
-      const float2 a01 = tc::ffma2(make_float2(v[q], v[q + 1]), cc, nm);
-      const float2 a23 = tc::ffma2(make_float2(v[q + 2], v[q + 3]), cc, nm);
+      const float2 a01 = tc::ffma2(make_float2(__uint_as_float(r[q]), __uint_as_float(r[q + 1])), cc, nm);
+      const float2 a23 = tc::ffma2(make_float2(__uint_as_float(r[q + 2]), __uint_as_float(r[q + 3])), cc, nm);
       s01 = tc::add2(s01, make_float2(tc::ex2(a01.x), tc::ex2(a01.y)));
       s23 = tc::add2(s23, make_float2(tc::ex2(a23.x), tc::ex2(a23.y)));
     }
-    const float s0 = s01.x, s1 = s01.y, s2 = s23.x, s3 = s23.y;
-    // a row with nothing visible yet keeps (-inf, 0); exp2(-inf - -inf) would be NaN
-    if (mn != -INFINITY) {
-      l = l * tc::ex2(m - mn) + ((s0 + s1) + (s2 + s3));
-      m = mn;
-    }
-    if (p + 1 < pe) tc::tmem_wait(nx);
-  };
-  tc::tmem_ld32_async(taddr, ra);
-  tc::tmem_wait(ra);
+  });
+  return (s01.x + s01.y) + (s23.x + s23.y);
+}
+// Pass 1: the slice added to (reference m, sum l of exp2(c2 z - m)) of the row. A row
+// without a reference takes the maximum of its first chunk; a slice is then summed against
+// the reference as it stands, and only where the sum leaves its range (or is a NaN, or
+// there is still no reference) is the slice's maximum taken and the slice summed again.
+template <bool MASKED>
+__device__ __forceinline__ void p1_slice(uint32_t taddr, int pe, int lim, float c2, float& m, float& l) {
+  auto refer = [&](int chunks) {
+    float t = -INFINITY;
+    p1_chunks<MASKED>(taddr, chunks, lim, [&](const uint32_t(&r)[32]) {
 #pragma unroll
-  for (int p = 0; p < kChunks; p += 2) {
-    if (p < pe) chunk(ra, rb, p);
-    if (p + 1 < pe) chunk(rb, ra, p + 1);
+      for (int q = 0; q < 32; ++q) t = fmaxf(t, __uint_as_float(r[q]));
+    });
+    const float mb = t * c2;
+    if (mb > m + kRescaleTau) {
+      if (m != -INFINITY) l *= tc::ex2(m - mb);
+      m = mb;
+    }
+  };
+  if (__any_sync(0xffffffffu, m == -INFINITY && lim >= 0)) refer(1);
+  float sum = p1_sum<MASKED>(taddr, pe, lim, c2, m);
+  if (__any_sync(0xffffffffu, (m == -INFINITY && lim >= 0) || !(sum <= kRescaleSum))) {
+    refer(pe);
+    sum = p1_sum<MASKED>(taddr, pe, lim, c2, m);
   }
+  l += sum;
 }
 
-// Pass 2: sum of exp2(c2 * z - lse2[c]) over the columns c of a key. `nlse` holds
-// -lse2; a column that does not see the key carries -inf, which makes its term 0.
-__device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, float c2) {
-  uint32_t ra[32], rb[32];
+// Pass 2: sum of exp2(c2 * z - lse2[c]) over the columns c >= c0 of a key's slice. `nlse`
+// holds -lse2. Chunks before c0 are not looked at; the one it falls into reads -inf there.
+__device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, int c0, float c2) {
   // four partial sums (columns q mod 4), two per packed register
   float2 m01 = make_float2(0.f, 0.f), m23 = m01;
   const float2 cc = make_float2(c2, c2);
-  auto chunk = [&](uint32_t(&r)[32], uint32_t(&nx)[32], int p) {
-    if (p + 1 < kChunks) tc::tmem_ld32_async(taddr + (p + 1) * 32, nx);
+#pragma unroll 1
+  for (int p = c0 > 0 ? c0 >> 5 : 0; p < kChunks; ++p) {
+    uint32_t r[32];
+    tc::tmem_ld32_async(taddr + p * 32, r);
     const float4* l4 = reinterpret_cast<const float4*>(nlse + p * 32);
+    tc::tmem_wait(r);
+    if (c0 > p * 32) {
+#pragma unroll
+      for (int q = 0; q < 32; ++q) r[q] = (p * 32 + q >= c0) ? r[q] : 0xff800000u;
+    }
 #pragma unroll
     for (int q4 = 0; q4 < 8; ++q4) {
       const float4 lv = l4[q4];
@@ -302,31 +258,27 @@ __device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, flo
       m01 = tc::add2(m01, make_float2(tc::ex2(a01.x), tc::ex2(a01.y)));
       m23 = tc::add2(m23, make_float2(tc::ex2(a23.x), tc::ex2(a23.y)));
     }
-    if (p + 1 < kChunks) tc::tmem_wait(nx);
-  };
-  tc::tmem_ld32_async(taddr, ra);
-  tc::tmem_wait(ra);
-#pragma unroll
-  for (int p = 0; p < kChunks; p += 2) {
-    chunk(ra, rb, p);
-    chunk(rb, ra, p + 1);
   }
   return (m01.x + m01.y) + (m23.x + m23.y);
 }
 
 __device__ __forceinline__ void setup_sync(Sync& sy, int warp) {
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kP2Stages; ++s) {
-      tc::mbar_init(&sy.a_full[s], 1);
-      tc::mbar_init(&sy.a_empty[s], 1);
+    for (int s = 0; s < kStages; ++s) {
+      tc::mbar_init(&sy.k_full[s], 1);
+      tc::mbar_init(&sy.k_empty[s], 2);
     }
-    for (int s = 0; s < 2; ++s) {
-      tc::mbar_init(&sy.b_full[s], 1);
-      tc::mbar_init(&sy.b_empty[s], 1);
-      tc::mbar_init(&sy.acc_full[s], 1);
-      tc::mbar_init(&sy.acc_empty[s], kEpiWarps);
+    for (int t = 0; t < 2; ++t) {
+      tc::mbar_init(&sy.b_full[t], 1);
+      tc::mbar_init(&sy.b_empty[t], 1);
     }
-    tc::mbar_init(&sy.drain, 1);
+    for (int b = 0; b < 2; ++b)
+      for (int t = 0; t < 2; ++t) {
+        tc::mbar_init(&sy.acc_full[b][t], 1);
+        tc::mbar_init(&sy.acc_empty[b][t], kGroupWarps);
+      }
+    tc::mbar_init(&sy.drain[0], 1);
+    tc::mbar_init(&sy.drain[1], 1);
     sy.abort = 0;
     tc::fence_mbar_init();
   }
@@ -349,319 +301,297 @@ __device__ __forceinline__ void teardown(Sync& sy, int warp, uint32_t tmem, DevS
   if (threadIdx.x == 0 && sy.abort) record_error(st, AVTP_ERR_TIMEOUT, static_cast<int32_t>(blockIdx.x));
 }
 
+// ---------------------------------------------------------------- the two passes' common parts
+// Accumulator t (rows 128 t .. of the block) of the steps of parity b: 128 columns each.
+__device__ __forceinline__ uint32_t acc_col(int b, int t) { return static_cast<uint32_t>(b * 256 + t * 128); }
+
+// The row block of the walk's block, in halves of 128 rows (number nbl of the CTA's blocks):
+// a half is loaded as soon as its last product is done.
+template <int D>
+__device__ __forceinline__ bool load_block(unsigned char* sB, const CUtensorMap* mapQ, int g, int R0, uint32_t nbl,
+                                           Sync& sy) {
+  for (int t = 0; t < 2; ++t) {
+    if (nbl >= 1 && !tc::mbar_wait(&sy.b_empty[t], (nbl - 1) & 1)) return false;
+    tc::mbar_arrive_expect_tx(&sy.b_full[t], static_cast<uint32_t>(a_bytes(D)));
+    for (int ac = 0; ac < D / 64; ++ac)
+      tc::tma_load_3d(sB + ac * (kBlk * 128) + t * (kM * 128), mapQ, ac * 64, R0 + t * kM, g, &sy.b_full[t]);
+  }
+  return true;
+}
+// Key tile load number n: 128 keys of group g from packed position key0.
+template <int D>
+__device__ __forceinline__ bool load_keys(unsigned char* sK, const CUtensorMap* mapK, int g, int key0, uint32_t n,
+                                          Sync& sy) {
+  const int sk = n % kStages;
+  if (n >= kStages && !tc::mbar_wait(&sy.k_empty[sk], (n / kStages - 1) & 1)) return false;
+  tc::mbar_arrive_expect_tx(&sy.k_full[sk], static_cast<uint32_t>(a_bytes(D)));
+  for (int ac = 0; ac < D / 64; ++ac)
+    tc::tma_load_3d(sK + sk * a_bytes(D) + ac * (kM * 128), mapK, ac * 64, g, key0, &sy.k_full[sk]);
+  return true;
+}
+// Lets the copies in flight land before the CTA may exit.
+__device__ __forceinline__ void drain_loads(Sync& sy, uint32_t nk, uint32_t nbl) {
+  for (int t = 0; t < 2 && nbl >= 1; ++t) tc::mbar_wait(&sy.b_full[t], (nbl - 1) & 1);
+  for (uint32_t k = (nk >= kStages ? nk - kStages : 0); k < nk; ++k)
+    tc::mbar_wait(&sy.k_full[k % kStages], (k / kStages) & 1);
+}
+
+// The MMAs of half t of the block over a CTA's run, by one elected thread (the halves run on
+// two warps, each at the pace of its own epilogues, up to kStages key tiles apart). Pass 1
+// (the log-sum-exp) takes 128 rows as A and the key tile as B, pass 2 (the mass) the key
+// tile as A and 128 rows as B, into the accumulator of the half and the step's parity. The
+// next step's barriers are looked at before the commit ahead of them (behind it the look
+// outlasts the MMAs queued).
+template <int D, int PASS>
+__device__ __forceinline__ void issue_steps(int t, Walk<PASS> cur, int n_steps, uint32_t rows, uint32_t keys,
+                                            uint32_t tmem, Sync& sy) {
+  constexpr uint32_t idesc = tc::idesc_bf16(kM, kM);
+  constexpr uint32_t atomK = kM * 128, atomB = kBlk * 128;  // bytes per 64-element atom column
+  const uint32_t rt = rows + t * (kM * 128);
+  uint32_t nbl = 0;
+  bool new_seg = true, bad = false, k_seen = false, acc_seen = false;
+  auto wait = [&](uint64_t* bar, uint32_t parity, bool seen) {
+    if (!seen && !bad) bad = !tc::mbar_wait(bar, parity);
+  };
+#pragma unroll 1
+  for (int st = 0; st < n_steps && !bad; ++st) {
+    const int sk = st % kStages, b = st & 1;
+    if (t == 0) attn_stamp(PASS - 1, st, 1);
+    if (new_seg) wait(&sy.b_full[t], nbl++ & 1, false);
+    wait(&sy.k_full[sk], (st / kStages) & 1, k_seen);
+    // its previous use (step st - 2) must have been read out
+    if (st >= 2) wait(&sy.acc_empty[b][t], ((st >> 1) - 1) & 1, acc_seen);
+    if (t == 0) attn_stamp(PASS - 1, st, 2);
+    tc::fence_after_sync();
+    const uint32_t kt = keys + sk * static_cast<uint32_t>(a_bytes(D));
+    if (PASS == 1) tc::mma_rows<D>(tmem + acc_col(b, t), rt, atomB, kt, atomK, idesc);
+    else tc::mma_rows<D>(tmem + acc_col(b, t), kt, atomK, rt, atomB, idesc);
+    const bool more = st + 1 < n_steps;
+    acc_seen = st >= 1 && tc::mbar_test_wait(&sy.acc_empty[b ^ 1][t], (((st + 1) >> 1) - 1) & 1);
+    k_seen = more && tc::mbar_test_wait(&sy.k_full[(st + 1) % kStages], ((st + 1) / kStages) & 1);
+    tc::mma_commit(&sy.acc_full[b][t]);
+    tc::mma_commit(&sy.k_empty[sk]);
+    if (!more || cur.last_of_block()) tc::mma_commit(&sy.b_empty[t]);
+    new_seg = more && cur.next();
+    if (t == 0) attn_stamp(PASS - 1, st, 3);
+  }
+  if (bad) *static_cast<volatile int*>(&sy.abort) = 1;
+  // every MMA issued has completed once this arrives
+  tc::mma_commit(&sy.drain[t]);
+  tc::mbar_wait(&sy.drain[t], 0);
+}
+
 // ---------------------------------------------------------------- pass 1: log-sum-exp of every row
-// mapQ: Qt {d, rows, Hkv}, box 64 x 128 x 1; mapK: keys {d, Hkv, T}, box 64 x 1 x 256.
+// mapQ: Qt {d, rows, Hkv}, box 64 x 128 x 1; mapK: keys {d, Hkv, T}, box 64 x 1 x 128.
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 k_attn_lse(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK, AttnArgs a) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ Sync sy;
-  __shared__ float2 s_mrg[2][2][kM];  // [segment parity][A tile][row]: column half 1's (max, sum)
+  __shared__ float2 s_mrg[2][kBlk];  // [segment parity][row]: the odd steps' (reference, sum)
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int d = a.d;
-  unsigned char* sA = smem;  // A tile t at sA + t * a_bytes(d)
-  unsigned char* sB[2] = {smem + 2 * a_bytes(d), smem + 2 * a_bytes(d) + b_bytes(d)};
+  unsigned char* sB = smem;                // the block's rows
+  unsigned char* sK = smem + b_bytes(D);  // key tile s at sK + s * a_bytes(D)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t atomA = kM * 128, atomB = kN * 128;  // bytes per 64-element atom column
 
-  pdl_wait();
-  pdl_trigger();
-  if (!a.st->layout_ok) return;
-  const int NB = a.blk_cu[a.R];
-  const int F1 = a.meta[0], C1 = a.meta[1];
-  const int64_t total = static_cast<int64_t>(a.Hkv) * F1;
-  const int64_t f_begin = static_cast<int64_t>(blockIdx.x) * C1;
-  if (f_begin >= total) return;
-  const int n_steps = static_cast<int>(min(f_begin + C1, total) - f_begin);
-
+  // TMEM first: the next kernel's CTAs, which also allocate all of it, may start on this SM
+  // from the trigger on, and wait for this grid with it
   setup_sync(sy, warp);
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem = sy.tmem;
   volatile int* abort_flag = &sy.abort;
-  FlatCursor cur;
-  cur.init(f_begin, F1, a.p1s_cu, NB);
+  const int4 start = a.cta_start[blockIdx.x];
+  const int n_steps = a.st->layout_ok ? start.w : 0;
+  Walk<1> cur{};
+  if (n_steps > 0) cur.init(a, start);
 
-  if (warp == kTmaWarp) {
+  if (n_steps == 0) {
+    // nothing to do (or a layout that did not validate)
+  } else if (warp == kTmaWarp) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       tc::tma_prefetch_map(&mapQ);
       tc::tma_prefetch_map(&mapK);
-      uint32_t na = 0, nb = 0;  // A (block) loads and B (key tile) loads issued so far
-      int key_base = 0;
+      uint32_t nk = 0, nbl = 0;  // key tile loads and block loads issued so far
       bool new_seg = true;
       for (int st = 0; st < n_steps && !*abort_flag; ++st) {
-        if (new_seg) {
-          if (na >= 1 && !tc::mbar_wait(&sy.a_empty[0], (na - 1) & 1)) { *abort_flag = 1; break; }
-          const Seg s = seg_of(a, cur.g, cur.b);
-          tc::mbar_arrive_expect_tx(&sy.a_full[0], static_cast<uint32_t>(2 * a_bytes(d)));
-          for (int t = 0; t < 2; ++t)
-            for (int ac = 0; ac < d / 64; ++ac)
-              tc::tma_load_3d(sA + t * a_bytes(d) + ac * atomA, &mapQ, ac * 64, static_cast<int>(s.R0) + t * kM,
-                              cur.g, &sy.a_full[0]);
-          ++na;
-          key_base = a.cu[s.r];
-        }
-        const int sb = nb & 1;
-        if (nb >= 2 && !tc::mbar_wait(&sy.b_empty[sb], ((nb >> 1) - 1) & 1)) { *abort_flag = 1; break; }
-        tc::mbar_arrive_expect_tx(&sy.b_full[sb], static_cast<uint32_t>(b_bytes(d)));
-        for (int ac = 0; ac < d / 64; ++ac)
-          tc::tma_load_3d(sB[sb] + ac * atomB, &mapK, ac * 64, cur.g, key_base + cur.j * kN, &sy.b_full[sb]);
+        if (!load_keys<D>(sK, &mapK, cur.g, cur.blk.key0 + cur.j * kM, nk, sy)) { *abort_flag = 1; break; }
         attn_stamp(0, st, 0);
-        ++nb;
-        new_seg = st + 1 < n_steps && cur.next(a.p1s_cu, NB);
-      }
-      // let the copies in flight land before the CTA may exit
-      if (na >= 1) tc::mbar_wait(&sy.a_full[0], (na - 1) & 1);
-      for (uint32_t k = (nb >= 2 ? nb - 2 : 0); k < nb; ++k) tc::mbar_wait(&sy.b_full[k & 1], (k >> 1) & 1);
-    }
-  } else if (warp == kMmaWarp) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16(kM, kN);
-      uint32_t na = 0, nb = 0;
-      bool new_seg = true, stop = false;
-      for (int st = 0; st < n_steps && !stop && !*abort_flag; ++st) {
-        attn_stamp(0, st, 1);
+        ++nk;
         if (new_seg) {
-          if (!tc::mbar_wait(&sy.a_full[0], na & 1)) { *abort_flag = 1; break; }
-          ++na;
+          if (!load_block<D>(sB, &mapQ, cur.g, cur.blk.R0, nbl, sy)) { *abort_flag = 1; break; }
+          ++nbl;
         }
-        const int sb = nb & 1;
-        if (!tc::mbar_wait(&sy.b_full[sb], (nb >> 1) & 1)) { *abort_flag = 1; break; }
-        for (int t = 0; t < 2; ++t) {
-          // accumulator t: its previous use (step nb - 1) must have been read out
-          if (nb >= 1 && !tc::mbar_wait(&sy.acc_empty[t], (nb - 1) & 1)) { *abort_flag = 1; stop = true; break; }
-          if (t == 0) attn_stamp(0, st, 2);
-          tc::fence_after_sync();
-          tc::mma_rows(tmem + t * kN, tc::smem_u32(sA + t * a_bytes(d)), atomA, tc::smem_u32(sB[sb]), atomB, d, idesc);
-          tc::mma_commit(&sy.acc_full[t]);
-        }
-        if (stop) break;
-        tc::mma_commit(&sy.b_empty[sb]);
-        attn_stamp(0, st, 3);
-        ++nb;
-        const bool more = st + 1 < n_steps;
-        if (!more || cur.last_of_block()) tc::mma_commit(&sy.a_empty[0]);
-        new_seg = more && cur.next(a.p1s_cu, NB);
+        new_seg = st + 1 < n_steps && cur.next();
       }
-      // every MMA issued has completed once this arrives
-      tc::mma_commit(&sy.drain);
-      tc::mbar_wait(&sy.drain, 0);
+      drain_loads(sy, nk, nbl);
     }
+  } else if (warp >= kMmaWarp) {
+    // ------------------------------------------------------------ MMA issuers: rows (A) x keys (B)
+    if (tc::elect_one())
+      issue_steps<D, 1>(warp - kMmaWarp, cur, n_steps, tc::smem_u32(sB), tc::smem_u32(sK), tmem, sy);
   } else {
-    // ------------------------------------------------------------ epilogue (8 warps)
-    // Warp w reads TMEM lanes 32(w%4)..+31 (its rows of both A tiles) and columns
-    // 128(w/4)..+127 of both accumulators; the two column halves of a row meet in
-    // shared memory when the row's partial is written.
-    const int quad = warp & 3, half = warp >> 2;
-    const int lrow = quad * 32 + lane;  // row of each A tile = TMEM lane
-    const uint32_t tbase = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * (kN / 2);
+    // ------------------------------------------------------------ epilogue, 4 warps per accumulator
+    // Warp w reads TMEM lanes 32(w%4)..+31 (its rows of A tile t) of the accumulators of the
+    // steps of parity b; the two parities of a row meet in shared memory when the row's
+    // partial is written.
+    const int quad = warp & 3, t = (warp >> 2) & 1, b = warp >> 3;
+    const int lrow = t * kM + quad * 32 + lane;  // row of the block
+    const uint32_t taddr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + acc_col(b, t);
     const float c2 = a.c2;
-    // After a timeout (abort_flag) the epilogue keeps walking the same steps, skipping
-    // every wait and TMEM read, so that its named barriers still line up.
-    int key_base = 0, qpos0 = -1, qpos1 = -1, par = 0;
-    bool new_seg = true;
-    float2* dst0 = nullptr;          // this row's partial (A tile 0, 1) of the current block
-    float2* dst1 = nullptr;
-    float m0 = -INFINITY, l0 = 0.f, m1 = -INFINITY, l1 = 0.f;  // running max and sum, log2 domain
+    // After a wait that gave up (ok false) the warp keeps walking the same steps, skipping
+    // every wait and TMEM read, so that the named barriers still line up.
+    const int F1 = a.meta[0], C1 = a.meta[1];
+    int qpos = -1, par = 0;
+    bool new_seg = true, ok = true;
+    float2* dst = nullptr;         // this row's partial of the current block
+    float m = -INFINITY, l = 0.f;  // reference and sum, log2 domain
     for (int st = 0; st < n_steps; ++st) {
       if (new_seg) {
-        const Seg s = seg_of(a, cur.g, cur.b);
-        key_base = a.cu[s.r];
-        const int64_t F0 = static_cast<int64_t>(cur.g) * F1 + a.p1s_cu[cur.b];
+        const int64_t F0 = static_cast<int64_t>(cur.g) * F1 + cur.blk.s1;
         const int slot = static_cast<int>(blockIdx.x - F0 / C1);
-        const int64_t row0 = s.R0 + lrow, row1 = s.R0 + kM + lrow;
-        float2* base = a.p1_part + (static_cast<int64_t>(cur.g * NB + cur.b) * kBlk + lrow) * kAttnMaxChunks + slot;
-        qpos0 = row0 < s.R1 ? a.text_idx[row0 / a.G] : -1;
-        qpos1 = row1 < s.R1 ? a.text_idx[row1 / a.G] : -1;
-        dst0 = row0 < s.R1 ? base : nullptr;
-        dst1 = row1 < s.R1 ? base + static_cast<int64_t>(kM) * kAttnMaxChunks : nullptr;
-        m0 = m1 = -INFINITY;
-        l0 = l1 = 0.f;
+        const bool live = lrow < cur.blk.rows;
+        qpos = live ? a.text_idx[(cur.blk.R0 + lrow) / a.G] : -1;
+        dst = live ? a.p1_part + (static_cast<int64_t>(cur.g * cur.NB + cur.b) * kBlk + lrow) * kAttnMaxChunks + slot
+                   : nullptr;
+        m = -INFINITY;
+        l = 0.f;
       }
-#pragma unroll 1
-      for (int t = 0; t < 2; ++t) {
-        bool ok = !__any_sync(0xffffffffu, *abort_flag != 0);
-        if (ok && !tc::mbar_wait_warp(&sy.acc_full[t], st & 1)) {
+      if ((st & 1) == b) {
+        if (ok && !tc::mbar_wait_warp(&sy.acc_full[b][t], (st >> 1) & 1)) {
           if (lane == 0) *abort_flag = 1;
           ok = false;
         }
-        if (t == 0 && warp == 0 && lane == 0) attn_stamp(0, st, 4);
+        if (warp == 0 && lane == 0) attn_stamp(0, st, 4);
         tc::fence_after_sync();
-        // columns 0..lim of this warp's half are visible to the row
-        const int lim = (t ? qpos1 : qpos0) - (key_base + cur.j * kN + half * (kN / 2));
+        // columns 0..lim are visible to the row
+        const int lim = qpos - (cur.blk.key0 + cur.j * kM);
         const int lim_max = __reduce_max_sync(0xffffffffu, lim);
         if (ok && lim_max >= 0) {
-          const uint32_t taddr = tbase + t * kN;
-          float mt = t ? m1 : m0, lt = t ? l1 : l0;
-          if (__all_sync(0xffffffffu, lim >= kHalf - 1)) {
-            p1_slice<false>(taddr, kChunks, lim, c2, mt, lt);
+          if (__all_sync(0xffffffffu, lim >= kM - 1)) {
+            p1_slice<false>(taddr, kChunks, lim, c2, m, l);
           } else {
             // 32-column chunks 0 .. pe-1 hold a visible column for some lane
-            p1_slice<true>(taddr, min(kChunks, (lim_max >> 5) + 1), lim, c2, mt, lt);
+            p1_slice<true>(taddr, min(kChunks, (lim_max >> 5) + 1), lim, c2, m, l);
           }
-          if (t) { m1 = mt; l1 = lt; } else { m0 = mt; l0 = lt; }
         }
         tc::fence_before_sync();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&sy.acc_empty[t]);
-        if (t == 1 && warp == 0 && lane == 0) attn_stamp(0, st, 5);
+        if (lane == 0) tc::mbar_arrive(&sy.acc_empty[b][t]);
+        if (warp == 0 && lane == 0) attn_stamp(0, st, 5);
       }
       const bool more = st + 1 < n_steps;
       if (!more || cur.last_of_block()) {
-        // the block ends here for this CTA: merge the column halves and write the partial
+        // the block ends here for this CTA: merge the step parities and write the partial
         par ^= 1;
-        if (half == 1) {
-          s_mrg[par][0][lrow] = make_float2(m0, l0);
-          s_mrg[par][1][lrow] = make_float2(m1, l1);
-        }
+        if (b == 1) s_mrg[par][lrow] = make_float2(m, l);
         bar_epi();
-        if (half == 0) {
-          auto merge = [&](float m, float l, float2 o, float2* dst) {
-            const float M = fmaxf(m, o.x);
-            const float L = (M == -INFINITY) ? 0.f : l * tc::ex2(m - M) + o.y * tc::ex2(o.x - M);
-            *dst = make_float2(M, L);
-          };
-          if (dst0 != nullptr) merge(m0, l0, s_mrg[par][0][lrow], dst0);
-          if (dst1 != nullptr) merge(m1, l1, s_mrg[par][1][lrow], dst1);
+        if (b == 0 && dst != nullptr) {
+          const float2 o = s_mrg[par][lrow];
+          const float M = fmaxf(m, o.x);
+          const float L = (M == -INFINITY) ? 0.f : l * tc::ex2(m - M) + o.y * tc::ex2(o.x - M);
+          *dst = make_float2(M, L);
         }
       }
-      new_seg = more && cur.next(a.p1s_cu, NB);
+      new_seg = more && cur.next();
     }
   }
   teardown(sy, warp, tmem, a.st);
 }
 
 // ---------------------------------------------------------------- pass 2: probability mass of every visual key
-// mapK: keys {d, Hkv, T}, box 64 x 1 x 128; mapQ: Qt {d, rows, Hkv}, box 64 x 256 x 1.
+// mapK: keys {d, Hkv, T}, box 64 x 1 x 128; mapQ: Qt {d, rows, Hkv}, box 64 x 128 x 1.
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 k_attn_mass(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapQ, AttnArgs a) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ Sync sy;
-  __shared__ __align__(16) float s_lse[2][kBlk];  // -lse2, [block parity][row of the block]
-  // key masses of the last steps, per column half, flushed to the accumulator every
-  // kMassWindow steps (global atomics inside the step loop would be waited for by the
+  __shared__ __align__(16) float s_lse[2][2][kBlk];  // -lse2, [step parity][block parity][row of the block]
+  // key masses of the last steps of a parity, per row half, flushed to the accumulator every
+  // kMassWindow of them (global atomics inside the step loop would be waited for by the
   // next step's TMEM fence)
-  __shared__ float s_mass[kMassWindow][2][kM];
-  __shared__ int s_tile[kMassWindow], s_nk[kMassWindow];
+  __shared__ float s_mass[2][kMassWindow][2][kM];
+  __shared__ int s_tile[2][kMassWindow], s_nk[2][kMassWindow];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int d = a.d;
-  unsigned char* sB = smem;  // the block's rows
-  unsigned char* sA0 = smem + b_bytes(d);  // key tile s at sA0 + s * a_bytes(d)
+  unsigned char* sB = smem;                // the block's rows
+  unsigned char* sK = smem + b_bytes(D);  // key tile s at sK + s * a_bytes(D)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t atomA = kM * 128, atomB = kN * 128;
 
-  pdl_wait();
-  pdl_trigger();
-  if (!a.st->layout_ok) return;
-  const int NB = a.blk_cu[a.R];
-  const int F1 = a.meta[0], C1 = a.meta[1], F2 = a.meta[2], C2 = a.meta[3];
-  const int64_t total = static_cast<int64_t>(a.Hkv) * F2;
-  const int64_t f_begin = static_cast<int64_t>(blockIdx.x) * C2;
-  if (f_begin >= total) return;
-  const int n_steps = static_cast<int>(min(f_begin + C2, total) - f_begin);
-
+  // TMEM first: the next kernel's CTAs, which also allocate all of it, may start on this SM
+  // from the trigger on, and wait for this grid with it
   setup_sync(sy, warp);
+  pdl_trigger();
+  pdl_wait();
   const uint32_t tmem = sy.tmem;
   volatile int* abort_flag = &sy.abort;
-  FlatCursor cur;
-  cur.init(f_begin, F2, a.p2t_cu, NB);
+  const int4 start = a.cta_start[gridDim.x + blockIdx.x];
+  const int n_steps = a.st->layout_ok ? start.w : 0;
+  Walk<2> cur{};
+  if (n_steps > 0) cur.init(a, start);
 
-  if (warp == kTmaWarp) {
+  if (n_steps == 0) {
+    // nothing to do (or a layout that did not validate)
+  } else if (warp == kTmaWarp) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       tc::tma_prefetch_map(&mapQ);
       tc::tma_prefetch_map(&mapK);
-      uint32_t na = 0, nbl = 0;  // key tile loads and block loads issued so far
+      uint32_t nk = 0, nbl = 0;  // key tile loads and block loads issued so far
       bool new_seg = true;
-      Seg s{};
-      TileCursor tile{};
+      int key0 = a.tile_info[cur.blk.tile0 + cur.j].x;
       for (int st = 0; st < n_steps && !*abort_flag; ++st) {
-        if (new_seg) {
-          if (nbl >= 1 && !tc::mbar_wait(&sy.b_empty[0], (nbl - 1) & 1)) { *abort_flag = 1; break; }
-          s = seg_of(a, cur.g, cur.b);
-          tc::mbar_arrive_expect_tx(&sy.b_full[0], static_cast<uint32_t>(b_bytes(d)));
-          for (int ac = 0; ac < d / 64; ++ac)
-            tc::tma_load_3d(sB + ac * atomB, &mapQ, ac * 64, static_cast<int>(s.R0), cur.g, &sy.b_full[0]);
-          ++nbl;
-          tile.init(a, s, cur.j);
-        } else {
-          tile.next(a, s);
-        }
-        const int sa = na % kP2Stages;
-        if (na >= kP2Stages && !tc::mbar_wait(&sy.a_empty[sa], ((na / kP2Stages) - 1) & 1)) { *abort_flag = 1; break; }
-        tc::mbar_arrive_expect_tx(&sy.a_full[sa], static_cast<uint32_t>(a_bytes(d)));
-        for (int ac = 0; ac < d / 64; ++ac)
-          tc::tma_load_3d(sA0 + sa * a_bytes(d) + ac * atomA, &mapK, ac * 64, cur.g, tile.kp0, &sy.a_full[sa]);
+        if (!load_keys<D>(sK, &mapK, cur.g, key0, nk, sy)) { *abort_flag = 1; break; }
         attn_stamp(1, st, 0);
-        ++na;
-        new_seg = st + 1 < n_steps && cur.next(a.p2t_cu, NB);
-      }
-      if (nbl >= 1) tc::mbar_wait(&sy.b_full[0], (nbl - 1) & 1);
-      for (uint32_t k = (na >= kP2Stages ? na - kP2Stages : 0); k < na; ++k)
-        tc::mbar_wait(&sy.a_full[k % kP2Stages], (k / kP2Stages) & 1);
-    }
-  } else if (warp == kMmaWarp) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = tc::idesc_bf16(kM, kN);
-      uint32_t na = 0, nbl = 0;
-      bool new_seg = true;
-      for (int st = 0; st < n_steps && !*abort_flag; ++st) {
-        attn_stamp(1, st, 1);
-        if (new_seg) {
-          if (!tc::mbar_wait(&sy.b_full[0], nbl & 1)) { *abort_flag = 1; break; }
+        ++nk;
+        const int g = cur.g, R0 = cur.blk.R0;
+        const bool load = new_seg;
+        new_seg = st + 1 < n_steps && cur.next();
+        if (st + 1 < n_steps) key0 = a.tile_info[cur.blk.tile0 + cur.j].x;
+        if (load) {
+          if (!load_block<D>(sB, &mapQ, g, R0, nbl, sy)) { *abort_flag = 1; break; }
           ++nbl;
         }
-        const int sa = na % kP2Stages;
-        if (!tc::mbar_wait(&sy.a_full[sa], (na / kP2Stages) & 1)) { *abort_flag = 1; break; }
-        const int t = na & 1;  // accumulator of this step
-        if (na >= 2 && !tc::mbar_wait(&sy.acc_empty[t], ((na >> 1) - 1) & 1)) { *abort_flag = 1; break; }
-        attn_stamp(1, st, 2);
-        tc::fence_after_sync();
-        tc::mma_rows(tmem + t * kN, tc::smem_u32(sA0 + sa * a_bytes(d)), atomA, tc::smem_u32(sB), atomB, d, idesc);
-        tc::mma_commit(&sy.a_empty[sa]);
-        tc::mma_commit(&sy.acc_full[t]);
-        attn_stamp(1, st, 3);
-        ++na;
-        const bool more = st + 1 < n_steps;
-        if (!more || cur.last_of_block()) tc::mma_commit(&sy.b_empty[0]);
-        new_seg = more && cur.next(a.p2t_cu, NB);
       }
-      tc::mma_commit(&sy.drain);
-      tc::mbar_wait(&sy.drain, 0);
+      drain_loads(sy, nk, nbl);
     }
+  } else if (warp >= kMmaWarp) {
+    // ------------------------------------------------------------ MMA issuers: keys (A) x rows (B)
+    if (tc::elect_one())
+      issue_steps<D, 2>(warp - kMmaWarp, cur, n_steps, tc::smem_u32(sB), tc::smem_u32(sK), tmem, sy);
   } else {
-    // ------------------------------------------------------------ epilogue (8 warps)
-    // Warp w reads TMEM lanes 32(w%4)..+31 (its keys) and columns 128(w/4)..+127 (rows
-    // of the block) of the step's accumulator; each column half adds its own share of a
-    // key's mass to the fixed-point accumulator.
-    const int quad = warp & 3, half = warp >> 2;
-    const int klane = quad * 32 + lane;  // key of the tile = TMEM lane
-    const int etid = threadIdx.x;        // 0 .. 255
-    const uint32_t tbase = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * (kBlk / 2);
+    // ------------------------------------------------------------ epilogue, 4 warps per accumulator
+    // Warp w reads TMEM lanes 32(w%4)..+31 (its keys) of the accumulators of row half `half`
+    // of the steps of parity t; the halves of a key's mass meet at the flush into the
+    // fixed-point accumulator.
+    const int quad = warp & 3, half = (warp >> 2) & 1, t = warp >> 3;
+    const int klane = quad * 32 + lane;                       // key of the tile = TMEM lane
+    const int etid = static_cast<int>(threadIdx.x) - t * kSetThreads;  // 0 .. 255
+    const uint32_t taddr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + acc_col(t, half);
     const float c2 = a.c2;
-    int par = 0, c1 = 0, img = -1;
-    float lse_own = INFINITY;  // lse2 of this thread's row of the block (row etid)
-    bool new_seg = true;
-    Seg s{};
-    TileCursor tile{};
-    for (int st = 0; st < n_steps; ++st) {
+    int par = 0, c1 = 0;
+    bool new_seg = true, ok = true;  // ok: see k_attn_lse
+    const int F1 = a.meta[0], C1 = a.meta[1];
+    int4 tile = make_int4(0, 0, 0, 0);
+    if (t == 1 && n_steps > 1) cur.next();
+    if (t < n_steps) tile = a.tile_info[cur.blk.tile0 + cur.j];
+    for (int st = t, w = 0; st < n_steps; st += 2) {
       if (new_seg) {
-        s = seg_of(a, cur.g, cur.b);
-        c1 = static_cast<int>(s.R1 - s.R0);  // rows of the block that belong to the request
-        const int g = cur.g, b = cur.b;
-        const int64_t row = s.R0 + etid;
-        lse_own = INFINITY;
-        if (row < s.R1) {
+        c1 = cur.blk.rows;
+        const int g = cur.g;
+        float lse_own = INFINITY;  // lse2 of this thread's row of the block (row etid)
+        if (etid < c1) {
+          const int64_t row = static_cast<int64_t>(cur.blk.R0) + etid;
           if (a.lse_rows != nullptr) {
             lse_own = a.lse_rows[static_cast<int64_t>(g) * a.rows + row];
           } else {
             // merge the row's pass-1 partials, eight loads in flight at a time
-            const int64_t F0 = static_cast<int64_t>(g) * F1 + a.p1s_cu[b];
-            const int steps = a.p1s_cu[b + 1] - a.p1s_cu[b];
+            const int64_t F0 = static_cast<int64_t>(g) * F1 + cur.blk.s1;
+            const int steps = cur.blk.n1;
             const int n = static_cast<int>((F0 + steps - 1) / C1 - F0 / C1) + 1;
-            const float2* src = a.p1_part + (static_cast<int64_t>(g * NB + b) * kBlk + etid) * kAttnMaxChunks;
+            const float2* src = a.p1_part + (static_cast<int64_t>(g * cur.NB + cur.b) * kBlk + etid) * kAttnMaxChunks;
             float M = -INFINITY, L = 0.f;
             for (int k0 = 0; k0 < n; k0 += 8) {
               float2 pk[8];
@@ -676,54 +606,46 @@ k_attn_mass(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
                 }
               }
             }
-            lse_own = M + __log2f(L);
+            lse_own = M + log2f(L);
           }
         }
-        tile.init(a, s, cur.j);
-        img = -1;
-      } else {
-        tile.next(a, s);
-      }
-      if (tile.i != img) {
-        // the -lse2 vector of this (block, image): -inf on rows whose query precedes the
-        // image, so that their terms vanish; double-buffered by parity
-        img = tile.i;
+        // rows past the request's carry -inf, which makes their terms vanish; thread etid's
+        // row is one that its own accumulator's threads read
         par ^= 1;
-        s_lse[par][etid] = (etid >= tile.c0) ? -lse_own : -INFINITY;
-        bar_epi();
+        s_lse[t][par][etid] = -lse_own;
+        bar_acc(t, half);
       }
-      const int t = st & 1;                                  // accumulator of this step
-      const uint32_t use = static_cast<uint32_t>(st) >> 1;  // its use count
-      bool ok = !__any_sync(0xffffffffu, *abort_flag != 0);
-      if (ok && !tc::mbar_wait_warp(&sy.acc_full[t], use & 1)) {
+      if (ok && !tc::mbar_wait_warp(&sy.acc_full[t][half], (static_cast<uint32_t>(st) >> 1) & 1)) {
         if (lane == 0) *abort_flag = 1;
         ok = false;
       }
       if (warp == 0 && lane == 0) attn_stamp(1, st, 4);
       tc::fence_after_sync();
-      // does this warp's column half hold a visible row? (CTA-uniform)
-      const bool any = tile.c0 < (half + 1) * kHalf && c1 > half * kHalf;
+      // first row of the block that sees the tile's image: its queries follow it
+      const int tile_id = cur.blk.tile0 + cur.j;
+      const int c0 = tile.z * a.G - cur.blk.R0;
+      // does this warp's row half hold a visible row? (uniform over its group)
+      const bool any = c0 < (half + 1) * kHalf && c1 > half * kHalf;
       float mass = 0.f;
-      if (ok && any) mass = p2_slice(tbase + t * kN, &s_lse[par][half * kHalf], c2);
+      if (ok && any) mass = p2_slice(taddr, &s_lse[t][par][half * kHalf], c0 - half * kHalf, c2);
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&sy.acc_empty[t]);
+      if (lane == 0) tc::mbar_arrive(&sy.acc_empty[t][half]);
       if (warp == 0 && lane == 0) attn_stamp(1, st, 5);
-      const int w = st % kMassWindow;
-      s_mass[w][half][klane] = mass;
+      s_mass[t][w][half][klane] = mass;
       if (etid == 0) {
-        s_tile[w] = tile.tile;
-        s_nk[w] = tile.nk;
+        s_tile[t][w] = tile_id;
+        s_nk[t][w] = tile.y;
       }
-      if (w == kMassWindow - 1 || st + 1 == n_steps) {
+      if (++w == kMassWindow || st + 2 >= n_steps) {
         // flush: one fixed-point integer add per (step, key), both column halves summed
         // in fp32 first (integer adds: the result does not depend on their order)
-        bar_epi();
-        for (int e = etid; e < (w + 1) * kM; e += kEpiWarps * 32) {
+        bar_set(t);
+        for (int e = etid; e < w * kM; e += kSetThreads) {
           const int ws = e / kM, k = e % kM;
-          if (k < s_nk[ws]) {
-            const float m = s_mass[ws][0][k] + s_mass[ws][1][k];
-            unsigned long long* dst = a.mass + static_cast<int64_t>(s_tile[ws]) * kM + k;
+          if (k < s_nk[t][ws]) {
+            const float m = s_mass[t][ws][0][k] + s_mass[t][ws][1][k];
+            unsigned long long* dst = a.mass + static_cast<int64_t>(s_tile[t][ws]) * kM + k;
             if (m <= 512.f) {  // at most one per row of the block
               atomicAdd(dst, static_cast<unsigned long long>(__float2ll_rn(m * static_cast<float>(1ull << kAttnMassFracBits))));
             } else {
@@ -731,9 +653,13 @@ k_attn_mass(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
             }
           }
         }
-        bar_epi();
+        bar_set(t);
+        w = 0;
       }
-      new_seg = st + 1 < n_steps && cur.next(a.p2t_cu, NB);
+      // two steps on, past the other parity's
+      new_seg = false;
+      for (int k = 0; k < 2 && st + 1 + k < n_steps; ++k) new_seg |= cur.next();
+      if (st + 2 < n_steps) tile = a.tile_info[cur.blk.tile0 + cur.j];
     }
   }
   teardown(sy, warp, tmem, a.st);
@@ -854,29 +780,22 @@ cudaError_t launch_score_attn(const avtp_layout_t& L, const avtp_score_args_t& s
   const AttnPlan plan = attn_plan(L, sa);
   static PerDevice attrs;
   cudaError_t ae = once_per_device(attrs, [](int, int*) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_lse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(lse_smem_bytes(128)));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_attn_mass, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(mass_smem_bytes(128)));
+    auto allow = [](auto kernel, size_t bytes) {
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    };
+    cudaError_t e = allow(k_attn_lse<128>, attn_smem_bytes(128));
+    if (e == cudaSuccess) e = allow(k_attn_lse<64>, attn_smem_bytes(64));
+    if (e == cudaSuccess) e = allow(k_attn_mass<128>, attn_smem_bytes(128));
+    if (e == cudaSuccess) e = allow(k_attn_mass<64>, attn_smem_bytes(64));
+    return e;
   });
   if (ae != cudaSuccess) return ae;
   DevStatus* st = ws_at<DevStatus>(ws, p.status);
   AttnArgs a{};
-  a.cu = L.cu_seqlens;
-  a.R = L.n_requests;
-  a.ist = L.img_start;
-  a.iln = L.img_len;
-  a.icu = L.img_cu;
-  a.NI = L.n_images;
-  a.T = L.n_tokens;
-  a.vis_cu = ws_at<int32_t>(ws, p.vis_cu);
   a.text_idx = ws_at<int32_t>(ws, p.text_idx);
-  a.text_cu = ws_at<int32_t>(ws, p.text_cu);
-  a.blk_cu = ws_at<int32_t>(ws, p.blk_cu);
-  a.p1s_cu = ws_at<int32_t>(ws, p.p1s_cu);
-  a.p2t_cu = ws_at<int32_t>(ws, p.p2t_cu);
-  a.ktile_cu = ws_at<int32_t>(ws, p.ktile_cu);
+  a.blk_info = ws_at<int4>(ws, p.blk_info);
+  a.tile_info = ws_at<int4>(ws, p.tile_info);
+  a.cta_start = ws_at<int4>(ws, p.cta_start);
   a.meta = ws_at<int32_t>(ws, p.meta);
   float* lse_rows = sa.lse != nullptr ? ws_at<float>(ws, p.lse_rows) : nullptr;
   a.lse_rows = lse_rows;
@@ -884,19 +803,15 @@ cudaError_t launch_score_attn(const avtp_layout_t& L, const avtp_score_args_t& s
   a.mass = ws_at<unsigned long long>(ws, p.mass);
   a.rows = plan.rows;
   a.G = plan.G;
-  a.Hkv = Hkv;
-  a.d = d;
   a.c2 = sa.softmax_scale * kLog2e;
   a.st = st;
   __nv_bfloat16* qt = ws_at<__nv_bfloat16>(ws, p.qt);
 
   // tensor maps: keys {d, Hkv, T} (token stride k_stride), packed queries {d, rows, Hkv}
-  CUtensorMap mk128, mk256, mq128, mq256;
+  CUtensorMap mk, mq;
   const uint64_t ks = static_cast<uint64_t>(sa.k_stride) * 2, qs = static_cast<uint64_t>(plan.rows) * d * 2;
-  if (!make_map(&mk128, sa.k, d, Hkv, L.n_tokens, static_cast<uint64_t>(d) * 2, ks, 1, kM) ||
-      !make_map(&mk256, sa.k, d, Hkv, L.n_tokens, static_cast<uint64_t>(d) * 2, ks, 1, kN) ||
-      !make_map(&mq128, qt, d, plan.rows, Hkv, static_cast<uint64_t>(d) * 2, qs, kM, 1) ||
-      !make_map(&mq256, qt, d, plan.rows, Hkv, static_cast<uint64_t>(d) * 2, qs, kBlk, 1))
+  if (!make_map(&mk, sa.k, d, Hkv, L.n_tokens, static_cast<uint64_t>(d) * 2, ks, 1, kM) ||
+      !make_map(&mq, qt, d, plan.rows, Hkv, static_cast<uint64_t>(d) * 2, qs, kM, 1))
     return cudaErrorInvalidValue;
 
   const int sms = plan.grid;
@@ -906,17 +821,18 @@ cudaError_t launch_score_attn(const avtp_layout_t& L, const avtp_score_args_t& s
     const int grid = static_cast<int>(want < 1 ? 1 : (want < cap ? want : cap));
     cudaError_t e = launch_kernel(k_attn_pack, dim3(grid), dim3(256), 0, s, /*pdl=*/true,
                                   static_cast<const __nv_bfloat16*>(sa.q), sa.q_stride, Hq, plan.G, d, a.text_idx,
-                                  a.text_cu, L.n_requests, plan.rows, qt, sa.lse, sa.lse_stride, lse_rows, a.mass,
+                                  static_cast<const int32_t*>(ws_at<int32_t>(ws, p.text_cu)), L.n_requests, plan.rows, qt, sa.lse, sa.lse_stride, lse_rows, a.mass,
                                   plan.n_ktiles_max * kM, static_cast<const DevStatus*>(st));
     if (e != cudaSuccess) return e;
   }
   if (sa.lse == nullptr) {
-    cudaError_t e = launch_kernel(k_attn_lse, dim3(sms), dim3(kThreads), lse_smem_bytes(d), s, /*pdl=*/true, mq128,
-                                  mk256, a);
+    cudaError_t e = launch_kernel(d == 128 ? k_attn_lse<128> : k_attn_lse<64>, dim3(sms), dim3(kThreads),
+                                  attn_smem_bytes(d), s, /*pdl=*/true, mq, mk, a);
     if (e != cudaSuccess) return e;
   }
   cudaError_t e =
-      launch_kernel(k_attn_mass, dim3(sms), dim3(kThreads), mass_smem_bytes(d), s, /*pdl=*/true, mk128, mq256, a);
+      launch_kernel(d == 128 ? k_attn_mass<128> : k_attn_mass<64>, dim3(sms), dim3(kThreads), attn_smem_bytes(d), s,
+                    /*pdl=*/true, mk, mq, a);
   if (e != cudaSuccess) return e;
   return launch_attn_finalize(L, sa, scores, img_sums, ws, p, plan, s);
 }

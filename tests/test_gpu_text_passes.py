@@ -1,0 +1,68 @@
+"""The text-attention criterion's tensor-core passes at their edges, against the fp64 oracle:
+key tiles of 128 and their remainders, row blocks of 256 and their halves, runs of a CTA that
+cross blocks, first visible rows inside a 32-row chunk, and a softmax reference that moves.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import avtp_oracle as O
+from paper_2608_26806_gb300 import avtp, synth
+from tests.gpu_util import assert_scores_close, bf16_dev, dev_layout, ensure_built
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    ensure_built()
+
+
+def _check(wl, scale=None, lse=None):
+    Hq, Hkv = wl.n_q_heads, wl.n_kv_heads
+    scale = wl.softmax_scale if scale is None else scale
+    L = dev_layout(wl.layout)
+    scores, sums = avtp.score(L, "text_attention", q=bf16_dev(wl.q), k=bf16_dev(wl.k), softmax_scale=scale, lse=lse,
+                              path="tensor")
+    torch.cuda.synchronize()
+    got = scores.cpu().numpy()
+    ref = O.score_text_attention(wl.layout, wl.q, wl.k, Hq, Hkv, scale)
+    assert_scores_close(got, ref, wl.layout.visual_mask())
+    assert np.array_equal(sums.cpu().numpy(), O.image_sums(wl.layout, got))
+
+
+_LAYOUTS = {
+    # image sizes about a key tile, one text token between the images (G rows each)
+    "tiles": [[("t", 2)] + [s for n in (1, 127, 128, 129, 255, 256, 257, 2) for s in (("i", n), ("t", 1))]],
+    # more row blocks than CTAs have steps: runs that cross several blocks
+    "blocks": [[("i", 130), ("t", 500)], [("t", 40), ("i", 3), ("t", 300)], [("i", 64), ("t", 129)]] * 3,
+    # requests whose rows end in the first half, at the half, and just past the block
+    "halves": [[("i", 200), ("t", n)] for n in (1, 31, 32, 33, 63, 64, 65, 128)],
+}
+
+
+@pytest.mark.parametrize("layout", sorted(_LAYOUTS))
+@pytest.mark.parametrize("heads", [(4, 1, 64), (8, 2, 128), (14, 2, 128)])
+def test_text_passes_edges(layout, heads):
+    Hq, Hkv, d = heads
+    _check(synth.make_custom(_LAYOUTS[layout], n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, hidden=64, seed=11,
+                             parts=("B",)))
+
+
+@pytest.mark.parametrize("growth", [40.0, -40.0])
+@pytest.mark.parametrize("heads", [(4, 2, 64), (8, 2, 128)])
+def test_text_passes_moving_reference(heads, growth):
+    """Logits that climb or fall by 40 over 500 keys move a row's reference again and again."""
+    Hq, Hkv, d = heads
+    wl = synth.make_custom([[("t", 3), ("i", 700), ("t", 90)], [("i", 260), ("t", 129)]], n_q_heads=Hq, n_kv_heads=Hkv,
+                           head_dim=d, hidden=64, seed=78, parts=("B",))
+    T = wl.layout.n_tokens
+    rng = np.random.default_rng(6)
+    ramp = growth * (np.arange(T) // 37) * 37 / 500.0
+    q = (np.full((T, Hq, d), 1.0 / d) + 0.002 * rng.standard_normal((T, Hq, d))).astype(np.float32)
+    k = (ramp[:, None, None] + rng.standard_normal((T, Hkv, d))).astype(np.float32)
+    wl.tensors["q"] = synth.f32_to_bf16_bits(q.reshape(T, -1)).reshape(T, Hq, d)
+    wl.tensors["k"] = synth.f32_to_bf16_bits(k.reshape(T, -1)).reshape(T, Hkv, d)
+    _check(wl, scale=1.0)
