@@ -428,6 +428,7 @@ constexpr int kTailKeys = (kKeyCap + kThreads - 33) / (kThreads - 32);
 // precedes the budget rule and the first histogram (which run side by side). The warm-up
 // run loads the same way from shared memory (generic loads serve both): while the scores
 // stream in, every global access waits behind them for microseconds.
+template <bool kMany>
 __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const AllocParams& ap, SelShared& sh,
                                                   const WarpAllocSmem& wsm, const WarpAllocSmem& wsm32,
                                                   const TailIn& in, bool dry) {
@@ -475,7 +476,7 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
     // ---- the budget rule, one warp
     int err;
     int k, before, total;
-    if (m <= 32) {
+    if (!kMany || m <= 32) {
 #ifdef AVTP_TIMELINE
       if (!dry && __shfl_sync(kFull, S_lane, 0) != INT64_MIN && lane == 0) timeline_stamp(a.st, kTlRuleBegin);
 #endif
@@ -597,10 +598,14 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
   if (tid == 0) timeline_stamp(a.st, kTlSelEnd);
 }
 
-// 184 registers: the tail runs without spilling (at 128 it spilled about 100 bytes a
-// thread, and local memory is slow to come back right after the scoring stream). One CTA
-// per SM, which is how the free SMs are used anyway.
-__global__ void __maxnreg__(184)
+// kMany: some request may have more than 32 images (the batch has more); the kernel for the
+// others carries none of that code. 184 and 240 registers: the tail runs without spilling
+// (at 128 it spilled about 100 bytes a thread, and local memory is slow to come back right
+// after the scoring stream; 96 bytes at 184 with the code for many images made the stage of
+// a 16-image request 0.8 us slower). One CTA per SM, which is how the free SMs are used
+// anyway.
+template <bool kMany>
+__global__ void __maxnreg__(kMany ? 240 : 184)
 k_alloc_select(SelectArgs a, AllocParams ap) {
   extern __shared__ __align__(16) unsigned char dsmem[];  // budget scratch for requests of > 32 images
   __shared__ __align__(16) unsigned char rule32[warp_alloc_smem_bytes(32)];  // ... and of at most 32
@@ -639,7 +644,7 @@ k_alloc_select(SelectArgs a, AllocParams ap) {
     int64_t nsum = 0, nbefore = 0;
     for (int j = lane; j < in.m; j += 32) {
       const int32_t nj = a.iln[in.i0 + j];
-      if (in.m > 32) wsm.n[j] = nj;
+      if (kMany && in.m > 32) wsm.n[j] = nj;
       else in.n_lane = nj;
       nsum += nj;
       nbefore += j < in.li ? nj : 0;
@@ -672,7 +677,7 @@ k_alloc_select(SelectArgs a, AllocParams ap) {
       pdl_trigger();
       if (tid == 0) timeline_stamp(a.st, kTlSelWaited);
     }
-    alloc_select_tail(a, ap, sh, wsm, wsm32, in, pass == 0);
+    alloc_select_tail<kMany>(a, ap, sh, wsm, wsm32, in, pass == 0);
   }
 }
 
@@ -727,16 +732,19 @@ cudaError_t launch_alloc_select(const avtp_layout_t& L, const int64_t* img_sums,
   // kernel can start on an SM where a scoring CTA still runs
   static PerDevice carveout;
   const cudaError_t ce = once_per_device(carveout, [](int, int*) {
-    return cudaFuncSetAttribute(k_alloc_select, cudaFuncAttributePreferredSharedMemoryCarveout,
+    const cudaError_t e = cudaFuncSetAttribute(k_alloc_select<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                               cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_alloc_select<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 cudaSharedmemCarveoutMaxShared);
   });
   if (ce != cudaSuccess) return ce;
   if (smem > 16 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_alloc_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_alloc_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
   }
-  return launch_kernel(k_alloc_select, dim3(L.n_images + L.n_requests), dim3(kThreads), smem, s, /*pdl=*/true, a,
+  return launch_kernel(ap.m_cap > 32 ? k_alloc_select<true> : k_alloc_select<false>, dim3(L.n_images + L.n_requests), dim3(kThreads), smem, s, /*pdl=*/true, a,
                        ap);
 }
 

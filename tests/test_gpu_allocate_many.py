@@ -1,0 +1,78 @@
+"""The budget rule for requests of more images than a warp has lanes, against the exact rule of
+the oracle, in avtp_allocate and in the fused stage: images per request about 32, 64, 96 and
+128 (the register form's lanes) and past them, with and without binding clamps, and with equal
+remainders at the largest-remainder cut.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import avtp_oracle as O
+from paper_2608_26806_gb300 import avtp, synth
+from tests.gpu_util import dev_layout, ensure_built
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    ensure_built()
+
+
+def _sums(rng, n, kind):
+    m = n.size
+    if kind == "mild":       # no clamp binds at r_base = 0.5
+        mean = rng.integers(2 ** 28, 2 ** 29, size=m)
+    elif kind == "strong":   # many images at the clamps
+        mean = rng.integers(-2 ** 33, 2 ** 34, size=m)
+    elif kind == "hot":      # a few far above the rest
+        mean = np.where(rng.random(m) < 0.05, 2 ** 32, 2 ** 26) + rng.integers(0, 2 ** 20, size=m)
+    else:                    # equal means: remainders tie between images of one size
+        mean = np.full(m, 2 ** 30)
+    return (mean * n).astype(np.int64)
+
+
+@pytest.mark.parametrize("m", [33, 63, 64, 65, 96, 97, 127, 128, 129, 200])
+@pytest.mark.parametrize("kind", ["mild", "strong", "hot", "equal"])
+@pytest.mark.parametrize("relative", [False, True])
+def test_allocate_many_images(m, kind, relative):
+    rng = np.random.default_rng(m * 7 + len(kind))
+    reqs = []
+    for mm in (m, 5, m - 1):
+        segs = [("t", 3)]
+        for _ in range(mm):
+            segs += [("i", int(rng.integers(1, 300)) if kind != "equal" else 37), ("t", int(rng.integers(0, 2)))]
+        reqs.append(segs)
+    lay = synth.Layout.from_segments(reqs)
+    n = lay.img_len.astype(np.int64)
+    S = _sums(rng, n, kind)
+    kr = np.array([0.5, 0.25, 0.125], dtype=np.float32)
+    L = dev_layout(lay)
+    for alpha in (1.0, 0.0, 3.0):
+        ref = O.allocate(lay, S, kr, alpha, 0.05, 0.95, relative)
+        budgets, out_cu = avtp.allocate(L, torch.from_numpy(S).cuda(), torch.from_numpy(kr).cuda(), alpha, 0.05, 0.95,
+                                        relative)
+        torch.cuda.synchronize()
+        assert np.array_equal(budgets.cpu().numpy(), ref["budgets"]), alpha
+        assert np.array_equal(out_cu.cpu().numpy(), ref["out_cu_seqlens"]), alpha
+
+
+@pytest.mark.parametrize("m", [33, 64, 100, 128, 140])
+def test_fused_stage_many_images(m):
+    """The same rule inside the fused stage, on the GPU's own scores."""
+    rng = np.random.default_rng(m)
+    segs = [("t", 4)]
+    for _ in range(m):
+        segs += [("i", int(rng.integers(1, 90))), ("t", 1)]
+    wl = synth.make_custom([segs, [("t", 2), ("i", 30)]], hidden=64, keep_ratio=0.33, seed=m, parts=("A",))
+    h_cur, h_prior = (torch.from_numpy(x.view(np.int16)).cuda().view(torch.bfloat16) for x in (wl.h_cur, wl.h_prior))
+    out = avtp.prune(dev_layout(wl.layout), "hidden_variation", keep_ratio=torch.from_numpy(wl.keep_ratio).cuda(),
+                     keep_ratio_host=wl.keep_ratio, rows={"hidden": h_cur}, h_cur=h_cur, h_prior=h_prior)
+    torch.cuda.synchronize()
+    assert avtp.read_device_status(out.workspace) == 0
+    ref = O.prune(wl.layout, keep_ratio=wl.keep_ratio, scores_f32=out.scores.cpu().numpy(), relative=False,
+                  rows={"hidden": wl.h_cur})
+    assert np.array_equal(out.budgets.cpu().numpy(), ref["budgets"])
+    assert np.array_equal(out.kept_idx.cpu().numpy(), ref["kept_idx"])
