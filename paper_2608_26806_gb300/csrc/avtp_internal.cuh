@@ -36,7 +36,7 @@ constexpr int kAttnMassFracBits = 40;    // fixed point of the per-key probabili
 // What the two passes need of a row block, laid out by the validation kernel (as two int4)
 // so that a walk over blocks takes one load where the prefix arrays would take a search.
 // Beside it: per key tile an int4 (first packed key, keys, text ordinals in the batch before
-// the token behind its image), and per CTA and pass an int4 (KV group, block, entry within
+// the token behind its image, request), and per CTA and pass an int4 (KV group, block, entry within
 // the block, steps of its run).
 struct AttnBlkInfo {
   int R0, rows;     // first row (of every KV group), rows
@@ -353,7 +353,7 @@ cudaError_t launch_score_attn(const avtp_layout_t& L, const avtp_score_args_t& s
                               int64_t* img_sums, void* ws, const WsPlan& p, cudaStream_t s);
 cudaError_t launch_score_narrow(const avtp_layout_t& L, const avtp_score_args_t& sa, float* scores, int64_t* img_sums,
                                 void* ws, const WsPlan& p, const AttnPlan& plan, cudaStream_t s);
-// Scores and fixed-point image sums from the per-key mass of either criterion-B path.
+// Scores and fixed-point image sums from the per-key mass of the tensor-core path.
 cudaError_t launch_attn_finalize(const avtp_layout_t& L, const avtp_score_args_t& sa, float* scores,
                                  int64_t* img_sums, void* ws, const WsPlan& p, const AttnPlan& plan, cudaStream_t s);
 

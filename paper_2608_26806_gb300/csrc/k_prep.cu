@@ -218,7 +218,7 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
         for (int t = t0; t < t1; ++t) {
           const int first = (t - t0) * kAttnTileM;
           ktile_img[t] = i;
-          tile_info[t] = make_int4(key0 + first, min(kAttnTileM, n - first), o_first, 0);
+          tile_info[t] = make_int4(key0 + first, min(kAttnTileM, n - first), o_first, r);
         }
       }
       // Pass 2 of block b: the key tiles of every image that at least one of the block's

@@ -702,23 +702,20 @@ k_attn_pack(const __nv_bfloat16* __restrict__ q, int64_t q_stride, int Hq, int G
 // the tile's fixed-point score sum added to its image's sum with one atomic.
 __global__ void __launch_bounds__(kM)
 k_attn_finalize(const unsigned long long* __restrict__ mass, const int32_t* __restrict__ ktile_cu,
-                const int32_t* __restrict__ ktile_img, int Hq, const int32_t* __restrict__ cu,
-                const int32_t* __restrict__ img_start, const int32_t* __restrict__ img_len,
-                const int32_t* __restrict__ img_req, const int32_t* __restrict__ text_cu, int NI, int last,
-                float* __restrict__ scores, int64_t* __restrict__ img_sums, const DevStatus* st) {
+                const int32_t* __restrict__ ktile_img, const int4* __restrict__ tile_info, int Hq,
+                const int32_t* __restrict__ text_cu, int NI, float* __restrict__ scores,
+                int64_t* __restrict__ img_sums, const DevStatus* st) {
   __shared__ long long s_part[kM / 32];
   pdl_wait();
   pdl_trigger();
   if (!st->layout_ok) return;
   for (int tile = blockIdx.x; tile < ktile_cu[NI]; tile += gridDim.x) {
     const int i = ktile_img[tile];
-    const int r = img_req[i];
-    const int o = (tile - ktile_cu[i]) * kM + static_cast<int>(threadIdx.x);  // key within the image
-    // the request's queries: its text tokens, or its last token alone
-    const int nq = last ? (cu[r + 1] > cu[r] ? 1 : 0) : text_cu[r + 1] - text_cu[r];
+    const int4 info = tile_info[tile];
     const unsigned long long m = mass[static_cast<int64_t>(tile) * kM + threadIdx.x];
+    const int nq = text_cu[info.w + 1] - text_cu[info.w];  // the request's queries
     long long fx = 0;
-    if (o < img_len[i]) {
+    if (static_cast<int>(threadIdx.x) < info.y) {
       float s = 0.f;
       if (nq > 0) {
         if (m & kMassNotFinite) {
@@ -728,7 +725,7 @@ k_attn_finalize(const unsigned long long* __restrict__ mass, const int32_t* __re
           s = s / static_cast<float>(static_cast<int64_t>(Hq) * nq);
         }
       }
-      scores[static_cast<int64_t>(cu[r]) + img_start[i] + o] = s;
+      scores[static_cast<int64_t>(info.x) + threadIdx.x] = s;
       fx = fixed_point_score(s);
     }
     fx = warp_sum(fx);
@@ -844,10 +841,9 @@ cudaError_t launch_attn_finalize(const avtp_layout_t& L, const avtp_score_args_t
   return launch_kernel(k_attn_finalize, dim3(grid3), dim3(kM), 0, s, /*pdl=*/true,
                        static_cast<const unsigned long long*>(ws_at<unsigned long long>(ws, p.mass)),
                        static_cast<const int32_t*>(ws_at<int32_t>(ws, p.ktile_cu)),
-                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.ktile_img)), sa.n_q_heads, L.cu_seqlens,
-                       L.img_start, L.img_len, static_cast<const int32_t*>(ws_at<int32_t>(ws, p.img_req)),
-                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.text_cu)), L.n_images,
-                       sa.query_set == AVTP_QUERIES_LAST ? 1 : 0, scores, img_sums,
+                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.ktile_img)),
+                       static_cast<const int4*>(ws_at<int4>(ws, p.tile_info)), sa.n_q_heads,
+                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.text_cu)), L.n_images, scores, img_sums,
                        static_cast<const DevStatus*>(ws_at<DevStatus>(ws, p.status)));
 }
 

@@ -66,3 +66,28 @@ def test_text_passes_moving_reference(heads, growth):
     wl.tensors["q"] = synth.f32_to_bf16_bits(q.reshape(T, -1)).reshape(T, Hq, d)
     wl.tensors["k"] = synth.f32_to_bf16_bits(k.reshape(T, -1)).reshape(T, Hkv, d)
     _check(wl, scale=1.0)
+
+
+@pytest.mark.parametrize("bad", [{"cu_seqlens": [0, 900, 200]}, {"cu_seqlens": [0, -5, 200]},
+                                 {"cu_seqlens": [7, 100, 200]}, {"img_start": [0, 180]}, {"img_len": [60, 0]}])
+def test_last_token_logits_beside_a_refused_layout(bad):
+    """The last-token logits run beside the layout's validation: offsets it refuses (decreasing,
+    negative, past the batch, spans outside their request) reach no memory outside the tensors
+    and leave the scores and sums untouched."""
+    lay = dict(cu_seqlens=[0, 100, 200], img_cu=[0, 1, 2], img_start=[0, 0], img_len=[60, 60])
+    good = avtp.Layout.from_host(**lay)
+    q = torch.randn(200, 8, 128, device="cuda").bfloat16()
+    k = torch.randn(200, 2, 128, device="cuda").bfloat16()
+    args = dict(q=q, k=k, query_set="last")
+    ws = avtp.new_workspace(avtp.workspace_size(good, "text_attention", **args) + 65536)
+    ref, _ = avtp.score(good, "text_attention", workspace=ws, **args)
+    host = {name: np.asarray({**lay, **bad}[name], dtype=np.int32) for name in lay}
+    dev = {name: torch.from_numpy(v.copy()).cuda() for name, v in host.items()}
+    # the host copies keep the good counts, as a caller's would
+    L = avtp.Layout(host=good.host, **dev)
+    scores = torch.full((200,), 7.0, device="cuda")
+    avtp.score(L, "text_attention", workspace=ws, scores=scores, **args)
+    assert avtp.read_device_status(ws) == avtp.ERR_DEVICE_INPUT
+    assert torch.all(scores == 7.0)
+    again, _ = avtp.score(good, "text_attention", workspace=ws, **args)
+    assert avtp.read_device_status(ws) == avtp.OK and torch.equal(ref, again)
