@@ -271,3 +271,41 @@ def test_forward_ignores_what_other_requests_hold(n, heads):
     mine = slice(5, 5 + n)
     _check_o(o.cpu().numpy()[mine], ref_o[mine], ref_abs[mine])
     np.testing.assert_allclose(lse.cpu().numpy()[:, mine], ref_lse[:, mine], rtol=RTOL, atol=ATOL)
+
+
+@pytest.mark.parametrize("bad", [{"cu_seqlens": [0, 400, 200, 600]}, {"cu_seqlens": [0, -5, 200, 600]},
+                                 {"cu_seqlens": [3, 100, 200, 600]}, {"cu_seqlens": [0, 100, 2 ** 30, 600]},
+                                 {"img_start": [0, 90, 0]}])
+@pytest.mark.parametrize("scores", [False, True])
+@pytest.mark.parametrize("repeat", [1, 14])
+def test_forward_beside_a_refused_layout(bad, scores, repeat):
+    """Up to 32 requests the forward runs beside the layout's validation (repeat 14: more, it
+    waits first): offsets validation refuses reach nothing outside the tensors, O, the LSE and
+    the scores stay untouched, and the next call is right again."""
+    lay = dict(cu_seqlens=[0, 100, 200, 600], img_cu=[0, 1, 2, 3], img_start=[0, 0, 0], img_len=[60, 60, 200])
+    if repeat > 1:  # the same three requests again and again
+        lay = dict(cu_seqlens=[0] + [600 * i + c for i in range(repeat) for c in (100, 200, 600)],
+                   img_cu=list(range(3 * repeat + 1)), img_start=[0] * 3 * repeat, img_len=[60, 60, 200] * repeat)
+        bad = {k: v + lay[k][len(v):] for k, v in bad.items()}
+    T = lay["cu_seqlens"][-1]
+    good = avtp.Layout.from_host(**lay)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    q = torch.randn(T, 8, 128, device="cuda", generator=gen).bfloat16()
+    k, v = (torch.randn(T, 2, 128, device="cuda", generator=gen).bfloat16() for _ in range(2))
+    c = avtp.ForwardCall(good, q=q, k=k, v=v, scores=scores)
+    c.run()
+    assert avtp.read_device_status(c.workspace) == avtp.OK
+    ref = [t.clone() for t in (c.o, c.lse)]
+    host = {name: np.asarray({**lay, **bad}[name], dtype=np.int32) for name in lay}
+    dev = {name: torch.from_numpy(x.copy()).cuda() for name, x in host.items()}
+    b = avtp.ForwardCall(avtp.Layout(host=good.host, **dev), q=q, k=k, v=v, scores=scores, workspace=c.workspace)
+    b.o.fill_(7.0), b.lse.fill_(7.0)
+    if scores:
+        b.scores.fill_(7.0)
+    b.run()
+    assert avtp.read_device_status(c.workspace) == avtp.ERR_DEVICE_INPUT
+    assert torch.all(b.o == 7.0) and torch.all(b.lse == 7.0) and (not scores or torch.all(b.scores == 7.0))
+    c.o.zero_(), c.lse.zero_()
+    c.run()
+    assert avtp.read_device_status(c.workspace) == avtp.OK
+    assert torch.equal(c.o, ref[0]) and torch.equal(c.lse, ref[1])
