@@ -1,7 +1,8 @@
 """The budget rule for requests of more images than a warp has lanes, against the exact rule of
 the oracle, in avtp_allocate and in the fused stage: images per request about 32, 64, 96 and
 128 (the register form's lanes) and past them, with and without binding clamps, and with equal
-remainders at the largest-remainder cut.
+remainders at the largest-remainder cut. And batches of about as many requests as a warp has
+lanes, some without images, where each image finds its request.
 """
 import numpy as np
 import pytest
@@ -76,3 +77,30 @@ def test_fused_stage_many_images(m):
                   rows={"hidden": wl.h_cur})
     assert np.array_equal(out.budgets.cpu().numpy(), ref["budgets"])
     assert np.array_equal(out.kept_idx.cpu().numpy(), ref["kept_idx"])
+
+
+@pytest.mark.parametrize("n_req", [1, 31, 32, 33, 70])
+@pytest.mark.parametrize("empty", ["none", "first", "last", "many"])
+def test_fused_stage_many_requests(n_req, empty):
+    """Each image's request, its neighbours and its place in the output, for batches about a warp wide."""
+    rng = np.random.default_rng(n_req)
+    reqs = []
+    for r in range(n_req):
+        bare = n_req > 1 and {"none": False, "first": r < 2 and r < n_req - 1, "last": r == n_req - 1,
+                              "many": r % 3 != 1}[empty]
+        segs = [("t", int(rng.integers(1, 9)))]
+        for _ in range(0 if bare else int(rng.integers(1, 4))):
+            segs += [("i", int(rng.integers(1, 60))), ("t", int(rng.integers(0, 3)))]
+        reqs.append(segs)
+    wl = synth.make_custom(reqs, hidden=64, keep_ratio=0.4, seed=n_req, parts=("A",))
+    h_cur, h_prior = (torch.from_numpy(x.view(np.int16)).cuda().view(torch.bfloat16) for x in (wl.h_cur, wl.h_prior))
+    out = avtp.prune(dev_layout(wl.layout), "hidden_variation", keep_ratio=torch.from_numpy(wl.keep_ratio).cuda(),
+                     keep_ratio_host=wl.keep_ratio, rows={"hidden": h_cur}, h_cur=h_cur, h_prior=h_prior)
+    torch.cuda.synchronize()
+    assert avtp.read_device_status(out.workspace) == 0
+    ref = O.prune(wl.layout, keep_ratio=wl.keep_ratio, scores_f32=out.scores.cpu().numpy(), relative=False,
+                  rows={"hidden": wl.h_cur})
+    assert np.array_equal(out.budgets.cpu().numpy(), ref["budgets"])
+    assert np.array_equal(out.kept_idx.cpu().numpy(), ref["kept_idx"])
+    kept = torch.from_numpy(ref["kept_idx"].astype(np.int64)).cuda()
+    assert torch.equal(out.outputs["hidden"].view(torch.int16), h_cur[kept].view(torch.int16))
