@@ -171,8 +171,8 @@ __device__ __forceinline__ float u128_to_float(u128 v) {
 // the budgets in sm.K; returns kExactFallback, having written nothing, when the partition
 // does not verify, or the largest-remainder cut falls among equal prefixes, or an image
 // would get more than one token. The general stage it stands in for keeps remainders of
-// three words in shared memory and ranks every image against every other: with it the fused
-// selection kernel of four requests of 64 images took 127 us, with this 41.
+// three words in shared memory and ranks every image against every other: with it the rule
+// and the selection of four requests of 64 images took 127 us in one kernel, with this 41.
 constexpr int kMultiLanes = 4;
 constexpr int kMultiImages = 32 * kMultiLanes;
 
@@ -457,19 +457,16 @@ static __device__ __noinline__ int warp_allocate(const WarpAllocSmem& sm, int m,
 static __device__ __noinline__ int64_t breakpoint_lambda32(int m, int64_t R, int64_t nl, bool has, int64_t target,
                                                     int64_t Rmin, int64_t Rmax, int64_t mx, int64_t mn) {
   int64_t lam;
-  auto G = [&](int64_t c) {
-    int64_t acc = 0;
-#pragma unroll 1
-    for (int j = 0; j < m; ++j) {
-      const int64_t Rj = __shfl_sync(0xffffffffu, R, j);
-      const int64_t nj = __shfl_sync(0xffffffffu, nl, j);
-      acc += nj * clamp64(Rj + c, Rmin, Rmax);
-    }
-    return acc;
-  };
-  // every lane evaluates its two breakpoints (all lanes take part in the shuffles)
+  // every lane evaluates G at its two breakpoints (all lanes take part in the shuffles)
   const int64_t cl = Rmin - R, ch = Rmax - R;
-  const int64_t gl = G(cl), gh = G(ch);
+  int64_t gl = 0, gh = 0;
+#pragma unroll 2
+  for (int j = 0; j < m; ++j) {
+    const int64_t Rj = __shfl_sync(0xffffffffu, R, j);
+    const int64_t nj = __shfl_sync(0xffffffffu, nl, j);
+    gl += nj * clamp64(Rj + cl, Rmin, Rmax);
+    gh += nj * clamp64(Rj + ch, Rmin, Rmax);
+  }
   int64_t c_lo = INT64_MIN, c_hi = INT64_MAX, g_lo = 0, g_hi = 0;
   if (has) {
     if (gl < target) { c_lo = cl; g_lo = gl; } else { c_hi = cl; g_hi = gl; }
@@ -642,20 +639,16 @@ __device__ __forceinline__ int exact32(bool has, int64_t S, int64_t n, int cls, 
   return AVTP_OK;
 }
 
-// A clamp binds: the grid's shift proposes the partition, checked exactly; the general
-// stage when that does not settle it. Out of line: fetched only when it runs.
-// The grid's shift: without clamps G is linear with slope N, so the smallest solution is
-// lambda0 = ceil((B * 2^40 - sum n_i R_i) / N); when no clamp binds at lambda0 - 1 or
-// lambda0, G is that line on [lambda0 - 1, lambda0] and lambda0 is exact. Otherwise the
-// breakpoints decide.
-static __device__ __noinline__ int warp_allocate32_clamped(const WarpAllocSmem& sm, int m, int64_t S, int32_t n,
-                                                           int64_t inv_n, int64_t B, int32_t N, int64_t inv_N,
-                                                           int64_t T, const RatioRule& rule, float alpha_f,
-                                                           float r_min_f, float r_max_f, int64_t Rb, int64_t Aa,
-                                                           int64_t mq, int64_t Mq, int32_t* k_out) {
+// The grid's shift, which proposes the partition when a clamp binds; *R_out is this lane's
+// ratio on the grid. Out of line: fetched only when it runs. Without clamps G is linear with
+// slope N, so the smallest solution is lambda0 = ceil((B * 2^40 - sum n_i R_i) / N); when no
+// clamp binds at lambda0 - 1 or lambda0, G is that line on [lambda0 - 1, lambda0] and lambda0
+// is exact. Otherwise the breakpoints decide.
+static __device__ __noinline__ int64_t grid_shift32(int m, int64_t S, int32_t n, int64_t inv_n, int64_t B, int32_t N,
+                                                    int64_t inv_N, int64_t T, const RatioRule& rule, int64_t Rmin,
+                                                    int64_t Rmax, int64_t* R_out) {
   const int lane = threadIdx.x & 31;
   const bool has = lane < m;
-  const int64_t Rmin = ratio_grid(r_min_f), Rmax = ratio_grid(r_max_f);
   // ---- ratios on the grid
   const int64_t avg = grid_mean(T, inv_N);
   const int64_t inv_avg = (rule.relative && avg != 0) ? recip62(avg > 0 ? avg : -avg) : 0;
@@ -680,33 +673,38 @@ static __device__ __noinline__ int warp_allocate32_clamped(const WarpAllocSmem& 
     }
   }
   if (!found) lam = breakpoint_lambda32(m, R, nl, has, target, Rmin, Rmax, mx, mn);
+  *R_out = R;
+  return lam;
+}
 
-  // ---- the exact stage on the grid's partition, in registers
-  const int64_t g = R + lam;
-  const int cls = g <= Rmin ? kClsLow : (g >= Rmax ? kClsHigh : kClsFree);
-  int32_t K = 0;
-  int err = rule.relative ? exact32<true>(has, S, n, cls, false, B, N, T, Rb, Aa, mq, Mq, &K)
-                          : exact32<false>(has, S, n, cls, false, B, N, T, Rb, Aa, mq, Mq, &K);
-  if (err == kExactFallback) {
-    if (has) {
-      sm.S[lane] = S;
-      sm.n[lane] = n;
-      sm.R[lane] = R;
-    }
-    __syncwarp();
-    err = exact_stage(sm, m, B, N, T, rule.r_base_f, alpha_f, r_min_f, r_max_f, rule.relative, lam, Rmin, Rmax);
-    K = has ? sm.K[lane] : 0;
-    __syncwarp();
+// The general stage for lane-held images (sm has 32 entries), where the register path's does
+// not settle the partition.
+static __device__ __noinline__ int general_stage32(const WarpAllocSmem& sm, int m, int64_t S, int32_t n, int64_t R,
+                                                   int64_t B, int32_t N, int64_t T, const RatioRule& rule,
+                                                   float alpha_f, float r_min_f, float r_max_f, int64_t lam,
+                                                   int64_t Rmin, int64_t Rmax, int32_t* k_out) {
+  const int lane = threadIdx.x & 31;
+  if (lane < m) {
+    sm.S[lane] = S;
+    sm.n[lane] = n;
+    sm.R[lane] = R;
   }
-  *k_out = K;
+  __syncwarp();
+  const int err =
+      exact_stage(sm, m, B, N, T, rule.r_base_f, alpha_f, r_min_f, r_max_f, rule.relative, lam, Rmin, Rmax);
+  *k_out = lane < m ? sm.K[lane] : 0;
+  __syncwarp();
   return err;
 }
 
 // The same rule for requests of at most 32 images, held in registers: lane j owns image
 // j (S_j, n_j in; its budget out). The partition with every image free (no clamp binds,
 // the common case) is checked exactly first; only when it fails does the grid search for
-// the shift (warp_allocate32_clamped), and only when that partition fails too does the
-// general stage run on sm (32 entries). Identical results and status to warp_allocate.
+// the shift (grid_shift32), and only when that partition fails too does the general stage
+// run on sm (32 entries). Both partitions are checked by one copy of the exact stage, in a
+// loop that is not unrolled: a second copy was fetched anew when a clamp bound, right behind
+// the scoring stream (the stage of eight images of 729 tokens, with a clamp binding, 33.8 ->
+// 33.0 us; of 16 images without one 43.7 -> 44.2). Identical results and status to warp_allocate.
 // inv_n = floor(2^62 / n_j) and inv_N = floor(2^62 / N) come from the caller, which
 // can take them before the sums are ready. Inlined: the fused selection kernel calls it
 // from one place for both its warm-up run and its real run, and a call would put the
@@ -721,15 +719,25 @@ __device__ __forceinline__ int warp_allocate32(const WarpAllocSmem& sm, int m, i
   const int64_t T = warp_sum(has ? S : int64_t(0));
   const int64_t Rb = units32(rule.r_base_f), Aa = units32(alpha_f), mq = units32(r_min_f), Mq = units32(r_max_f);
   int32_t K = 0;
-  // ---- first the partition of the common case, no clamp binding: no search needed
-  int err = rule.relative ? exact32<true>(has, S, n, kClsFree, true, B, N, T, Rb, Aa, mq, Mq, &K)
-                          : exact32<false>(has, S, n, kClsFree, true, B, N, T, Rb, Aa, mq, Mq, &K);
-  if (err != kExactFallback) {
-    *k_out = K;
-    return err;
+  int err, cls = kClsFree;
+  int64_t Rmin = 0, Rmax = 0, R = 0, lam = 0;
+#pragma unroll 1
+  for (int attempt = 0;; ++attempt) {
+    // ---- first the partition of the common case, no clamp binding: no search needed
+    err = rule.relative ? exact32<true>(has, S, n, cls, attempt == 0, B, N, T, Rb, Aa, mq, Mq, &K)
+                        : exact32<false>(has, S, n, cls, attempt == 0, B, N, T, Rb, Aa, mq, Mq, &K);
+    if (err != kExactFallback || attempt == 1) break;
+    // ---- then the grid's partition
+    Rmin = ratio_grid(r_min_f);
+    Rmax = ratio_grid(r_max_f);
+    lam = grid_shift32(m, S, n, inv_n, B, N, inv_N, T, rule, Rmin, Rmax, &R);
+    const int64_t g = R + lam;
+    cls = g <= Rmin ? kClsLow : (g >= Rmax ? kClsHigh : kClsFree);
   }
-  return warp_allocate32_clamped(sm, m, S, n, inv_n, B, N, inv_N, T, rule, alpha_f, r_min_f, r_max_f, Rb, Aa, mq,
-                                 Mq, k_out);
+  if (err == kExactFallback)
+    err = general_stage32(sm, m, S, n, R, B, N, T, rule, alpha_f, r_min_f, r_max_f, lam, Rmin, Rmax, &K);
+  *k_out = K;
+  return err;
 }
 
 }  // namespace avtp

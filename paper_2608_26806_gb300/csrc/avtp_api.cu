@@ -200,6 +200,7 @@ int device_sm_count() {
 constexpr int kMaxReserveSms = 32;
 
 int prune_reserve_sms(const avtp_layout_t& L) {
+  if (L.n_images > kFusedImages) return 1;  // k_allocate's
   if (L.n_tokens > 32768 || L.n_images < 1) return 0;
   const int64_t ctas = prune_warm_ctas(L);
   // one SM per selection CTA (its registers fill most of an SM; two on one SM slowed each
@@ -210,6 +211,7 @@ int prune_reserve_sms(const avtp_layout_t& L) {
 }
 
 int prune_warm_ctas(const avtp_layout_t& L) {
+  if (L.n_images > kFusedImages) return 1;  // k_allocate's
   if (L.n_tokens > 32768 || L.n_images < 1) return 0;
   const int64_t ctas = static_cast<int64_t>(L.n_images) + L.n_requests;
   return ctas <= kMaxWarmCtas ? static_cast<int>(ctas) : 0;

@@ -358,26 +358,32 @@ cudaError_t launch_attn_finalize(const avtp_layout_t& L, const avtp_score_args_t
                                  int64_t* img_sums, void* ws, const WsPlan& p, const AttnPlan& plan, cudaStream_t s);
 
 cudaError_t launch_allocate(const avtp_layout_t& L, const int64_t* img_sums, const avtp_alloc_args_t& aa,
-                            int32_t* budgets, void* ws, const WsPlan& p, cudaStream_t s);
+                            int32_t* budgets, void* ws, const WsPlan& p, cudaStream_t s, bool warm = false);  // warm: see k_allocate.cu
 
 cudaError_t launch_select(const avtp_layout_t& L, const float* scores, const int32_t* budgets,
                           const int32_t* out_cu_seqlens, int32_t* kept_idx, int64_t n_kept, void* ws,
-                          const WsPlan& p, cudaStream_t s);
+                          const WsPlan& p, cudaStream_t s, bool after_allocate = false);
 
-// Budget rule and selection in one kernel (the fused stage). Its first warm_ctas CTAs
-// run the code once on made-up data before waiting for the scores (see prune_reserve_sms).
+// Budget rule and selection of the fused stage. Up to kFusedImages images one kernel, in which
+// every image's CTA runs its request's rule; its first warm_ctas CTAs run the code once on
+// made-up data before waiting for the scores (see prune_reserve_sms). Beyond, k_allocate runs
+// the rule once per request (and warms up when warm_ctas > 0) and k_select selects, four CTAs
+// on an SM instead of the one that the rule's registers allow. Stage, one kernel against two:
+// 33 images of 729 tokens 136 / 91 us, 64 of 256 77 / 67, 127 in eight requests 139 / 132, 256
+// in four requests (1024 tokens each) 742 / 708; below, 16 images of 256-1024 tokens 44 / 52.
+constexpr int kFusedImages = 32;
 cudaError_t launch_alloc_select(const avtp_layout_t& L, const int64_t* img_sums, const avtp_alloc_args_t& aa,
                                 int32_t* budgets, const float* scores, const int32_t* out_cu_seqlens,
                                 int32_t* kept_idx, int64_t n_kept, void* ws, const WsPlan& p, cudaStream_t s,
                                 int warm_ctas = 0);
 
-// In avtp_prune with the hidden-variation criterion on a small batch, the scoring
-// kernel leaves prune_reserve_sms(L) SMs free so that the selection kernel's CTAs (one
+// In avtp_prune with the hidden-variation criterion on a small batch of at most kFusedImages
+// images, the scoring kernel leaves prune_reserve_sms(L) SMs free so that the selection kernel's CTAs (one
 // per image and one per request, one per SM) start while the scores stream in and warm
 // their instruction caches (prune_warm_ctas(L) of them run the code once on made-up data
 // first); 0 otherwise. Right after the scoring stream has swept L2 a cold run of the
 // budget rule and the selection takes several times longer. On large batches the
-// scoring time would grow instead.
+// scoring time would grow instead. Batches of more images leave one SM, to k_allocate.
 constexpr int kMaxWarmCtas = 96;
 int prune_reserve_sms(const avtp_layout_t& L);
 int prune_warm_ctas(const avtp_layout_t& L);

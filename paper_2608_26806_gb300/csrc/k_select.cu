@@ -12,11 +12,11 @@
 // position; kept positions are written in order after two block scans. The CTA
 // also writes the text run that follows its image.
 //
-// Two kernels: k_select takes the budgets as input (avtp_select); k_alloc_select
-// runs the budget rule of avtp_alloc.cuh for the image's request in warp 0 while
-// warps 1-7 stage the keys and build the first histogram, then selects
-// (avtp_prune). Everything that needs only the call's inputs is done before the
-// kernel waits for the scoring kernel, so it overlaps the scoring.
+// Two kernels of one tail: k_select takes the budgets as input (avtp_select, and avtp_prune
+// behind k_allocate); k_alloc_select runs the budget rule of avtp_alloc.cuh for the image's
+// request in warp 0 while warps 1-7 stage the keys and build the first histogram, then
+// selects (avtp_prune of up to kFusedImages images). Everything that needs only the call's
+// inputs is done before the kernel waits for the one before it, so it overlaps that one.
 #include "avtp_alloc.cuh"
 
 namespace avtp {
@@ -41,7 +41,6 @@ struct SelectArgs {
   int32_t* kept_idx;
   int64_t n_kept;
   const int32_t* vis_cu;
-  const int32_t* img_req;
   DevStatus* st;
 };
 
@@ -281,55 +280,6 @@ __device__ __forceinline__ bool select_from_first_pass(int n, int k, int64_t t0,
   return true;
 }
 
-// Stage the image's keys (when they fit) and find their range; all threads call.
-__device__ void stage_and_range(const float* __restrict__ sc, int n, bool stage, SelShared& sh, uint32_t* kmin_out,
-                                uint32_t* kmax_out) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t lo = 0xffffffffu, hi = 0u;
-  if (stage) {
-    uint32_t v[kPer];
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {  // all loads in flight at once
-      const int j = tid + q * kThreads;
-      v[q] = j < n ? rank_key(sc[j]) : 0u;
-    }
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int j = tid + q * kThreads;
-      if (j < n) {
-        sh.keys[j] = v[q];
-        lo = min(lo, v[q]);
-        hi = max(hi, v[q]);
-      }
-    }
-  } else {
-    for (int j = tid; j < n; j += kThreads) {
-      const uint32_t key = rank_key(sc[j]);
-      lo = min(lo, key);
-      hi = max(hi, key);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = min(lo, __shfl_xor_sync(kFull, lo, o));
-    hi = max(hi, __shfl_xor_sync(kFull, hi, o));
-  }
-  if (lane == 0) {
-    sh.wmin[warp] = lo;
-    sh.wmax[warp] = hi;
-  }
-  __syncthreads();
-  lo = sh.wmin[0];
-  hi = sh.wmax[0];
-#pragma unroll
-  for (int w = 1; w < kWarps; ++w) {
-    lo = min(lo, sh.wmin[w]);
-    hi = max(hi, sh.wmax[w]);
-  }
-  *kmin_out = lo;
-  *kmax_out = hi;
-}
-
 // Text before the first image of request r (the whole request if it has none).
 __device__ void leading_text(const SelectArgs& a, int r) {
   const int Tr = a.cu[r + 1] - a.cu[r];
@@ -342,81 +292,35 @@ __device__ void leading_text(const SelectArgs& a, int r) {
   for (int p = threadIdx.x; p < first; p += kThreads) a.kept_idx[base + p] = a.cu[r] + p;
 }
 
-__global__ void __launch_bounds__(kThreads)
-k_select(SelectArgs a, const int32_t* __restrict__ budgets) {
-  __shared__ SelShared sh;
-  pdl_wait();
-  pdl_trigger();
-  if (!a.st->layout_ok) return;
-  const int b = blockIdx.x;
-  if (b >= a.NI) {
-    leading_text(a, b - a.NI);
-    return;
-  }
-  const int i = b;
-  const int r = a.img_req[i];
-  const int i0 = a.icu[r], i1 = a.icu[r + 1];
-  int before = 0, total = 0, bad = 0;
-  for (int j = i0 + threadIdx.x; j < i1; j += kThreads) {
-    const int kj = budgets[j];
-    bad |= (kj < 0 || kj > a.iln[j]);
-    total += kj;
-    before += (j < i) ? kj : 0;
-  }
-  int sb, st, sbad;
-  block_incl_scan(before, sh.wsum, &sb);
-  block_incl_scan(total, sh.wsum, &st);
-  block_incl_scan(bad, sh.wsum, &sbad);
-  if (sbad) {
-    if (threadIdx.x == 0) record_error(a.st, AVTP_ERR_DEVICE_INPUT, i);
-    return;
-  }
-  const int Tr = a.cu[r + 1] - a.cu[r];
-  const int ntxt = Tr - (a.vis_cu[i1] - a.vis_cu[i0]);
-  if (a.out_cu[r] < 0 || a.out_cu[r + 1] - a.out_cu[r] != st + ntxt ||
-      static_cast<int64_t>(a.out_cu[r + 1]) > a.n_kept) {
-    if (threadIdx.x == 0) record_error(a.st, AVTP_ERR_DEVICE_INPUT, i);
-    return;
-  }
-  const int s0 = a.ist[i], n = a.iln[i], k = budgets[i];
-  const int64_t base = static_cast<int64_t>(a.out_cu[r]) + (s0 - (a.vis_cu[i] - a.vis_cu[i0])) + sb;
-  const int64_t t0 = static_cast<int64_t>(a.cu[r]) + s0;
-  const bool stage = n <= kKeyCap;
-  uint32_t kmin, kmax;
-  stage_and_range(a.scores + t0, n, stage, sh, &kmin, &kmax);
-  block_select(a.scores + t0, n, k, t0, base, a.kept_idx, sh, stage, kmin, kmax, false);
-  const int e = s0 + n;
-  const int nxt = (i + 1 < i1) ? a.ist[i + 1] : Tr;
-  for (int p = e + threadIdx.x; p < nxt; p += kThreads) a.kept_idx[base + k + (p - e)] = a.cu[r] + p;
-}
-
 struct AllocParams {
   const int64_t* img_sums;
   const float* keep_ratio;
   float alpha, r_min, r_max;
   int relative;
-  int32_t* budgets;  // output: each CTA writes its own image's budget
-  int m_cap;
+  int32_t* budgets;  // k_alloc_select's output: each CTA writes its own image's budget
   int warm_ctas;     // CTAs below this index warm their instruction cache before the wait
+  // k_select's inputs: the budgets, and (behind k_allocate) the requests' own, negative where
+  // the rule refused the request; NULL: not looked at
+  const int32_t* given;
+  const int32_t* req_budget;
 };
 
-// What a CTA of k_alloc_select knows before the scores exist (from the call's inputs).
+// What a CTA knows before it waits (from the call's inputs).
 struct TailIn {
   int r, i0, m, li;
   int32_t s0, n, nxt, Tr;
   int64_t t0;
-  // warp 0: the request's sizes and the scalars of the budget rule
+  // warp 0 of k_alloc_select: the request's sizes and the scalars of the budget rule
   int32_t N, n_lane, vis_before;
   int64_t B, inv_n, inv_N;
-  float kr;
   RatioRule rule;
 };
 
 // Keys of the CTA's image held per thread of warps 1..7 right after the wait.
 constexpr int kTailKeys = (kKeyCap + kThreads - 33) / (kThreads - 32);
 
-// Everything k_alloc_select does once the scores exist. The kernel runs it twice from one
-// copy of the code (a loop that is not unrolled): first with dry set, before the wait, on
+// Everything the two kernels do once the scores exist. k_alloc_select (kRule) runs it twice
+// from one copy of the code (a loop that is not unrolled): first with dry set, before the wait, on
 // whatever the buffers hold then (every index is in bounds for any contents; the sums are
 // replaced by equal made-up means, so that the budget rule takes its common path),
 // writing nothing to global memory; then for real. The dry run leaves exactly this code
@@ -428,10 +332,9 @@ constexpr int kTailKeys = (kKeyCap + kThreads - 33) / (kThreads - 32);
 // precedes the budget rule and the first histogram (which run side by side). The warm-up
 // run loads the same way from shared memory (generic loads serve both): while the scores
 // stream in, every global access waits behind them for microseconds.
-template <bool kMany>
+template <bool kRule>
 __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const AllocParams& ap, SelShared& sh,
-                                                  const WarpAllocSmem& wsm, const WarpAllocSmem& wsm32,
-                                                  const TailIn& in, bool dry) {
+                                                  const WarpAllocSmem& wsm32, const TailIn& in, bool dry) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const int r = in.r, i0 = in.i0, m = in.m, li = in.li;
@@ -442,7 +345,6 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
   // where the loads below read: the call's buffers, or shared stand-ins for the warm-up
   const float* sc = dry ? reinterpret_cast<const float*>(sh.keys) : a.scores + t0;
   const int32_t* status = dry ? sh.dry_status : &a.st->layout_ok;
-  const int64_t* sums = dry ? wsm32.S : ap.img_sums + i0;
   const int32_t* out_cu = dry ? sh.dry_out : a.out_cu + r;
   const bool stage = n <= kKeyCap;
 
@@ -450,9 +352,22 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
   const int layout_ok = *status;
   int64_t S_lane = 0;
   int32_t out_lo = 0, out_hi = 0;
+  int32_t k_lane = 0, n_lane = 0, refused = 0, vis_first = 0, vis_own = 0, vis_end = 0;
   uint32_t key[kTailKeys];
   if (warp == 0) {
-    if (image && lane < m && m <= 32) S_lane = sums[lane];
+    if constexpr (kRule) {
+      const int64_t* sums = dry ? wsm32.S : ap.img_sums + i0;
+      if (image && lane < m) S_lane = sums[lane];
+    } else if (image) {
+      if (lane < m) {
+        k_lane = ap.given[i0 + lane];
+        n_lane = a.iln[i0 + lane];
+      }
+      if (ap.req_budget != nullptr) refused = ap.req_budget[r] < 0 ? 1 : 0;
+      vis_first = a.vis_cu[i0];
+      vis_own = a.vis_cu[i0 + li];
+      vis_end = a.vis_cu[i0 + m];
+    }
     if (image) {
       out_lo = out_cu[0];
       out_hi = out_cu[1];
@@ -476,7 +391,8 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
     // ---- the budget rule, one warp
     int err;
     int k, before, total;
-    if (!kMany || m <= 32) {
+    int32_t vis_before, N;
+    if constexpr (kRule) {
 #ifdef AVTP_TIMELINE
       if (!dry && __shfl_sync(kFull, S_lane, 0) != INT64_MIN && lane == 0) timeline_stamp(a.st, kTlRuleBegin);
 #endif
@@ -486,18 +402,29 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
       k = __shfl_sync(kFull, K, li);
       before = static_cast<int>(__reduce_add_sync(kFull, static_cast<uint32_t>(lane < li ? K : 0)));
       total = static_cast<int>(__reduce_add_sync(kFull, static_cast<uint32_t>(lane < m ? K : 0)));
+      vis_before = in.vis_before;
+      N = in.N;
     } else {
-      for (int j = lane; j < m; j += 32) wsm.S[j] = dry ? (static_cast<int64_t>(wsm.n[j]) << 30) : ap.img_sums[i0 + j];
-      __syncwarp();
-      err = warp_allocate(wsm, m, in.B, in.N, in.kr, ap.alpha, ap.r_min, ap.r_max, ap.relative);
-      int bs = 0, ts = 0;
+      // the request's budgets, a lane per image and 32 images a round
+      uint32_t bs = 0, ts = 0, own = 0;
+      int bad = 0;
       for (int j = lane; j < m; j += 32) {
-        ts += wsm.K[j];
-        bs += j < li ? wsm.K[j] : 0;
+        if (j >= 32) {
+          k_lane = ap.given[i0 + j];
+          n_lane = a.iln[i0 + j];
+        }
+        bad |= (k_lane < 0 || k_lane > n_lane) ? 1 : 0;
+        ts += static_cast<uint32_t>(k_lane);
+        bs += j < li ? static_cast<uint32_t>(k_lane) : 0u;
+        if (j == li) own = static_cast<uint32_t>(k_lane);
       }
-      before = warp_sum(bs);
-      total = warp_sum(ts);
-      k = wsm.K[li];
+      before = static_cast<int>(__reduce_add_sync(kFull, bs));
+      total = static_cast<int>(__reduce_add_sync(kFull, ts));
+      err = __any_sync(kFull, bad) ? AVTP_ERR_DEVICE_INPUT : AVTP_OK;
+      if (refused) err = AVTP_ERR_RANGE;  // k_allocate recorded the request's error
+      k = static_cast<int>(__reduce_add_sync(kFull, own));
+      vis_before = vis_own - vis_first;
+      N = vis_end - vis_first;
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) sh.hist[0][lane * 8 + q] = 0;  // warp 0 takes no part in the first pass
@@ -509,8 +436,8 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
       sh.alloc_err = err;
       sh.out_lo = out_lo;
       sh.out_hi = out_hi;
-      sh.vis_before = in.vis_before;
-      sh.n_vis = in.N;
+      sh.vis_before = vis_before;
+      sh.n_vis = N;
     }
   } else {
     // ---- warps 1..7: stage the keys, find their range, build the first histogram
@@ -576,10 +503,12 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
   const int32_t olo = sh.out_lo, ohi = sh.out_hi, vis_b = sh.vis_before, Nv = sh.n_vis;
   if (!dry) {
     if (sh.alloc_err != AVTP_OK) {
-      if (tid == 0) record_error(a.st, sh.alloc_err, r);
+      if (tid == 0) record_error(a.st, sh.alloc_err, kRule ? r : i);
       return;
     }
-    if (tid == 0) ap.budgets[i] = k;
+    if constexpr (kRule) {
+      if (tid == 0) ap.budgets[i] = k;
+    }
     if (olo < 0 || ohi - olo != total + (Tr - Nv) || static_cast<int64_t>(ohi) > a.n_kept) {
       if (tid == 0) record_error(a.st, AVTP_ERR_DEVICE_INPUT, i);
       return;
@@ -598,77 +527,83 @@ __device__ __forceinline__ void alloc_select_tail(const SelectArgs& a, const All
   if (tid == 0) timeline_stamp(a.st, kTlSelEnd);
 }
 
-// kMany: some request may have more than 32 images (the batch has more); the kernel for the
-// others carries none of that code. 184 and 240 registers: the tail runs without spilling
-// (at 128 it spilled about 100 bytes a thread, and local memory is slow to come back right
-// after the scoring stream; 96 bytes at 184 with the code for many images made the stage of
-// a 16-image request 0.8 us slower). One CTA per SM, which is how the free SMs are used
-// anyway.
-template <bool kMany>
-__global__ void __maxnreg__(kMany ? 240 : 184)
+// The set-up of image b's CTA from the call's inputs only. The layout may not be validated
+// yet, so every index is clamped; nothing here is used unless the validation kernel accepts
+// the layout.
+__device__ __forceinline__ TailIn image_setup(const SelectArgs& a, int b, int lane) {
+  TailIn in{};
+  // Two rounds of loads: the image's own entries and, a lane per request, the requests'
+  // first images; then the request's entries. (A search of img_cu and what hangs on it took
+  // five, each a DRAM latency on the CTAs that start behind the scoring stream: a 16-image
+  // request's whole stage 48.4 -> 46.6 us.) Beyond 32 requests the search stands in.
+  const int32_t s0 = a.ist[b], n0 = a.iln[b], after = b + 1 < a.NI ? a.ist[b + 1] : 0;
+  if (a.R <= 32) {
+    const int32_t first = lane < a.R ? a.icu[lane] : 0, end = lane < a.R ? a.icu[lane + 1] : 0;
+    const unsigned at_or_before = __ballot_sync(kFull, lane < a.R && first <= b);
+    in.r = max(31 - __clz(at_or_before), 0);
+    in.i0 = min(max(__shfl_sync(kFull, first, in.r), 0), a.NI);
+    in.m = min(max(__shfl_sync(kFull, end, in.r), in.i0), a.NI) - in.i0;
+  } else {
+    in.r = upper_index(a.icu, a.R, b);
+    in.i0 = min(max(a.icu[in.r], 0), a.NI);
+    in.m = min(max(a.icu[in.r + 1], in.i0), a.NI) - in.i0;
+  }
+  if (in.m > 0) {
+    in.li = min(max(b - in.i0, 0), in.m - 1);
+    const int32_t cu_r = a.cu[in.r];
+    in.Tr = a.cu[in.r + 1] - cu_r;
+    in.s0 = s0;
+    in.n = n0;
+    in.nxt = (in.li + 1 < in.m) ? after : in.Tr;
+    in.t0 = static_cast<int64_t>(cu_r) + in.s0;
+  }
+  // a span outside the scores (a malformed layout, reported by the validation kernel)
+  // is never read, not even by the dry run
+  if (in.t0 < 0 || in.n < 0 || in.t0 + in.n > a.T) {
+    in.t0 = 0;
+    in.n = 0;
+  }
+  return in;
+}
+
+// Budgets given: no rule, so few registers and four CTAs on an SM. The runtime's choice of
+// shared memory against L1: with all of it as shared memory (as k_alloc_select asks) the
+// gather behind this kernel was slower, 127 images of 256 tokens 139 us against 133.
+__global__ void __launch_bounds__(kThreads, 4)
+k_select(SelectArgs a, AllocParams ap) {
+  __shared__ SelShared sh;
+  const int b = blockIdx.x;
+  TailIn in{};
+  if (b < a.NI) in = image_setup(a, b, threadIdx.x & 31);
+  pdl_wait();
+  pdl_trigger();
+  alloc_select_tail<false>(a, ap, sh, WarpAllocSmem{}, in, false);
+}
+
+// 184 registers: the tail runs without spilling (at 128 it spilled about 100 bytes a thread,
+// and local memory is slow to come back right after the scoring stream). One CTA per SM,
+// which is how the free SMs are used anyway.
+__global__ void __maxnreg__(184)
 k_alloc_select(SelectArgs a, AllocParams ap) {
-  extern __shared__ __align__(16) unsigned char dsmem[];  // budget scratch for requests of > 32 images
-  __shared__ __align__(16) unsigned char rule32[warp_alloc_smem_bytes(32)];  // ... and of at most 32
+  __shared__ __align__(16) unsigned char rule32[warp_alloc_smem_bytes(32)];  // budget scratch
   __shared__ SelShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   if (tid == 0) timeline_stamp(a.st, kTlSelBegin);
-  const WarpAllocSmem wsm = carve_warp_alloc(dsmem, ap.m_cap);
   const WarpAllocSmem wsm32 = carve_warp_alloc(rule32, 32);
 
-  // ---- set-up from the call's inputs only, overlapped with the scoring kernel.
-  // The layout is not validated yet, so every index is clamped; nothing here is
-  // used unless the validation kernel accepts the layout.
+  // ---- set-up, overlapped with the scoring kernel
   TailIn in{};
-  if (b < a.NI) {
-    // Two rounds of loads: the image's own entries and, a lane per request, the requests'
-    // first images; then the request's entries. (A search of img_cu and what hangs on it took
-    // five, each a DRAM latency on the CTAs that start behind the scoring stream: a 16-image
-    // request's whole stage 48.4 -> 46.6 us.) Beyond 32 requests the search stands in.
-    const int32_t s0 = a.ist[b], n0 = a.iln[b], after = b + 1 < a.NI ? a.ist[b + 1] : 0;
-    if (a.R <= 32) {
-      const int32_t first = lane < a.R ? a.icu[lane] : 0, end = lane < a.R ? a.icu[lane + 1] : 0;
-      const unsigned at_or_before = __ballot_sync(kFull, lane < a.R && first <= b);
-      in.r = max(31 - __clz(at_or_before), 0);
-      in.i0 = min(max(__shfl_sync(kFull, first, in.r), 0), a.NI);
-      in.m = min(min(max(__shfl_sync(kFull, end, in.r), in.i0), a.NI) - in.i0, ap.m_cap);
-    } else {
-      in.r = upper_index(a.icu, a.R, b);
-      in.i0 = min(max(a.icu[in.r], 0), a.NI);
-      in.m = min(min(max(a.icu[in.r + 1], in.i0), a.NI) - in.i0, ap.m_cap);
-    }
-    if (in.m > 0) {
-      in.li = min(max(b - in.i0, 0), in.m - 1);
-      const int32_t cu_r = a.cu[in.r];
-      in.Tr = a.cu[in.r + 1] - cu_r;
-      in.s0 = s0;
-      in.n = n0;
-      in.nxt = (in.li + 1 < in.m) ? after : in.Tr;
-      in.t0 = static_cast<int64_t>(cu_r) + in.s0;
-    }
-    // a span outside the scores (a malformed layout, reported by the validation kernel)
-    // is never read, not even by the dry run
-    if (in.t0 < 0 || in.n < 0 || in.t0 + in.n > a.T) {
-      in.t0 = 0;
-      in.n = 0;
-    }
-  }
+  if (b < a.NI) in = image_setup(a, b, lane);
   if (warp == 0 && b < a.NI) {
-    int64_t nsum = 0, nbefore = 0;
-    for (int j = lane; j < in.m; j += 32) {
-      const int32_t nj = a.iln[in.i0 + j];
-      if (kMany && in.m > 32) wsm.n[j] = nj;
-      else in.n_lane = nj;
-      nsum += nj;
-      nbefore += j < in.li ? nj : 0;
-    }
-    in.N = static_cast<int32_t>(warp_sum(nsum));
-    in.vis_before = static_cast<int32_t>(warp_sum(nbefore));
-    in.kr = ap.keep_ratio[in.r];
+    if (lane < in.m) in.n_lane = a.iln[in.i0 + lane];
+    in.N = static_cast<int32_t>(warp_sum(static_cast<int64_t>(in.n_lane)));
+    in.vis_before = static_cast<int32_t>(warp_sum(static_cast<int64_t>(lane < in.li ? in.n_lane : 0)));
+    const float kr = ap.keep_ratio[in.r];
     // B_r = floor(r_base * N_vis + 0.5), each operation rounded once
     in.B = static_cast<int64_t>(
-        floor(__dadd_rn(__dmul_rn(static_cast<double>(in.kr), static_cast<double>(in.N)), 0.5)));
-    in.rule = make_ratio_rule(in.kr, ap.alpha, ap.relative);
+        floor(__dadd_rn(__dmul_rn(static_cast<double>(kr), static_cast<double>(in.N)), 0.5)));
+    in.rule = make_ratio_rule(kr, ap.alpha, ap.relative);
     in.inv_N = recip62(in.N);
     in.inv_n = recip62(in.n_lane);
   }
@@ -690,7 +625,7 @@ k_alloc_select(SelectArgs a, AllocParams ap) {
       pdl_trigger();
       if (tid == 0) timeline_stamp(a.st, kTlSelWaited);
     }
-    alloc_select_tail<kMany>(a, ap, sh, wsm, wsm32, in, pass == 0);
+    alloc_select_tail<true>(a, ap, sh, wsm32, in, pass == 0);
   }
 }
 
@@ -709,7 +644,6 @@ SelectArgs make_args(const avtp_layout_t& L, const float* scores, const int32_t*
   a.kept_idx = kept_idx;
   a.n_kept = n_kept;
   a.vis_cu = ws_at<int32_t>(ws, p.vis_cu);
-  a.img_req = ws_at<int32_t>(ws, p.img_req);
   a.st = ws_at<DevStatus>(ws, p.status);
   return a;
 }
@@ -718,17 +652,33 @@ SelectArgs make_args(const avtp_layout_t& L, const float* scores, const int32_t*
 
 cudaError_t launch_select(const avtp_layout_t& L, const float* scores, const int32_t* budgets,
                           const int32_t* out_cu_seqlens, int32_t* kept_idx, int64_t n_kept, void* ws,
-                          const WsPlan& p, cudaStream_t s) {
+                          const WsPlan& p, cudaStream_t s, bool after_allocate) {
   const SelectArgs a = make_args(L, scores, out_cu_seqlens, kept_idx, n_kept, ws, p);
-  return launch_kernel(k_select, dim3(L.n_images + L.n_requests), dim3(kThreads), 0, s, /*pdl=*/true, a, budgets);
+  AllocParams ap{};
+  ap.given = budgets;
+  ap.req_budget = after_allocate ? ws_at<int32_t>(ws, p.req_budget) : nullptr;
+  return launch_kernel(k_select, dim3(L.n_images + L.n_requests), dim3(kThreads), 0, s, /*pdl=*/true, a, ap);
 }
 
 cudaError_t launch_alloc_select(const avtp_layout_t& L, const int64_t* img_sums, const avtp_alloc_args_t& aa,
                                 int32_t* budgets, const float* scores, const int32_t* out_cu_seqlens,
                                 int32_t* kept_idx, int64_t n_kept, void* ws, const WsPlan& p, cudaStream_t s,
                                 int warm_ctas) {
+  if (L.n_images > kFusedImages) {
+    const cudaError_t e = launch_allocate(L, img_sums, aa, budgets, ws, p, s, /*warm=*/warm_ctas > 0);
+    if (e != cudaSuccess) return e;
+    return launch_select(L, scores, budgets, out_cu_seqlens, kept_idx, n_kept, ws, p, s, /*after_allocate=*/true);
+  }
+  // same shared-memory configuration as the scoring kernels, so that a CTA of this
+  // kernel can start on an SM where a scoring CTA still runs
+  static PerDevice carveout;
+  const cudaError_t ce = once_per_device(carveout, [](int, int*) {
+    return cudaFuncSetAttribute(k_alloc_select, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                cudaSharedmemCarveoutMaxShared);
+  });
+  if (ce != cudaSuccess) return ce;
   const SelectArgs a = make_args(L, scores, out_cu_seqlens, kept_idx, n_kept, ws, p);
-  AllocParams ap;
+  AllocParams ap{};
   ap.img_sums = img_sums;
   ap.keep_ratio = aa.keep_ratio;
   ap.alpha = aa.alpha;
@@ -737,28 +687,7 @@ cudaError_t launch_alloc_select(const avtp_layout_t& L, const int64_t* img_sums,
   ap.relative = aa.relative;
   ap.budgets = budgets;
   ap.warm_ctas = warm_ctas;
-  ap.m_cap = L.n_images < kMaxImagesPerRequest ? L.n_images : kMaxImagesPerRequest;
-  if (ap.m_cap < 1) ap.m_cap = 1;
-  // the budget scratch is only used for requests of more than 32 images
-  const size_t smem = ap.m_cap > 32 ? warp_alloc_smem_bytes(ap.m_cap) : 0;
-  // same shared-memory configuration as the scoring kernels, so that a CTA of this
-  // kernel can start on an SM where a scoring CTA still runs
-  static PerDevice carveout;
-  const cudaError_t ce = once_per_device(carveout, [](int, int*) {
-    const cudaError_t e = cudaFuncSetAttribute(k_alloc_select<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                               cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_alloc_select<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                cudaSharedmemCarveoutMaxShared);
-  });
-  if (ce != cudaSuccess) return ce;
-  if (smem > 16 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_alloc_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
-  return launch_kernel(ap.m_cap > 32 ? k_alloc_select<true> : k_alloc_select<false>, dim3(L.n_images + L.n_requests), dim3(kThreads), smem, s, /*pdl=*/true, a,
-                       ap);
+  return launch_kernel(k_alloc_select, dim3(L.n_images + L.n_requests), dim3(kThreads), 0, s, /*pdl=*/true, a, ap);
 }
 
 }  // namespace avtp

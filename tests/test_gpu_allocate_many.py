@@ -60,7 +60,7 @@ def test_allocate_many_images(m, kind, relative):
         assert np.array_equal(out_cu.cpu().numpy(), ref["out_cu_seqlens"]), alpha
 
 
-@pytest.mark.parametrize("m", [33, 64, 100, 128, 140])
+@pytest.mark.parametrize("m", [30, 31, 32, 33, 64, 100, 128, 140])
 def test_fused_stage_many_images(m):
     """The same rule inside the fused stage, on the GPU's own scores."""
     rng = np.random.default_rng(m)
