@@ -1,7 +1,7 @@
 // Step 2 as its own kernel (avtp_allocate): one warp per request runs the budget
 // rule of avtp_alloc.cuh (paper §3.3.3 adaptive keep ratio, App. A.2 clamps) and
-// writes the request's budgets: the register form (a lane per image) for requests of up
-// to 32 images, the shared-memory form beyond. avtp_prune of more than kFusedImages images
+// writes the request's budgets: a lane per image for requests of up to 32 images,
+// four or eight images a lane up to 256, shared memory beyond. avtp_prune of more than kFusedImages images
 // runs it between the scores and k_select.
 // Latency and instruction fetches bound it: right behind the scoring stream, which sweeps L2,
 // a cold run of the rule takes 15-25 us, most of it fetching code. With warm the kernel, which

@@ -1,6 +1,6 @@
 """The budget rule for requests of more images than a warp has lanes, against the exact rule of
-the oracle, in avtp_allocate and in the fused stage: images per request about 32, 64, 96 and
-128 (the register form's lanes) and past them, with and without binding clamps, and with equal
+the oracle, in avtp_allocate and in the fused stage: images per request about 32, 64, 96,
+128 and 256 (the register form's lanes) and past them, with and without binding clamps, and with equal
 remainders at the largest-remainder cut. And batches of about as many requests as a warp has
 lanes, some without images, where each image finds its request.
 """
@@ -35,7 +35,7 @@ def _sums(rng, n, kind):
     return (mean * n).astype(np.int64)
 
 
-@pytest.mark.parametrize("m", [33, 63, 64, 65, 96, 97, 127, 128, 129, 200])
+@pytest.mark.parametrize("m", [33, 63, 64, 65, 96, 97, 127, 128, 129, 200, 255, 256, 257])
 @pytest.mark.parametrize("kind", ["mild", "strong", "hot", "equal"])
 @pytest.mark.parametrize("relative", [False, True])
 def test_allocate_many_images(m, kind, relative):
@@ -60,7 +60,7 @@ def test_allocate_many_images(m, kind, relative):
         assert np.array_equal(out_cu.cpu().numpy(), ref["out_cu_seqlens"]), alpha
 
 
-@pytest.mark.parametrize("m", [30, 31, 32, 33, 64, 100, 128, 140])
+@pytest.mark.parametrize("m", [30, 31, 32, 33, 64, 100, 128, 140, 256, 257])
 def test_fused_stage_many_images(m):
     """The same rule inside the fused stage, on the GPU's own scores."""
     rng = np.random.default_rng(m)
