@@ -331,7 +331,7 @@ def run_ours(args, world, rank, local):
                                   query_set="last")
         prog = time_progressive(args, wl, L, h_cur, h_prior, pos, stream, flush, torch, avtp, world, dev)
         fwd = time_forward(args, wl, L, bf16, stream, flush, torch, avtp, world, dev)
-    variants = time_variants(args, call, stream, flush, torch, avtp, 4 if crit == "hidden_variation" else 7)
+    variants = time_variants(args, call, stream, flush, torch, avtp, stage_launches(wl, crit))
     clocks = sampler.stop() if sampler else None
     barrier(world)
     step_ms = [a.elapsed_time(b) for a, b in outer]
@@ -384,7 +384,7 @@ def run_ours(args, world, rank, local):
         "roofline": roof,
         "e2e": e2e,
         "e2e_pipelined": e2e_pipe,
-        "gpu_launches": K * (4 if crit == "hidden_variation" else 7) + variants["launches"],
+        "gpu_launches": K * stage_launches(wl, crit) + variants["launches"],
         "clocks": clocks,
     }
     hbm_s, bf16_s, _ = measured_peaks()
@@ -441,7 +441,7 @@ def run_ours(args, world, rank, local):
             "with_scores_us": round(with_b * 1e3, 2), "with_scores_p50_us": res["with_scores"]["p50_us"],
             "criterion_b_marginal_us": round((with_b - plain) * 1e3, 2),
             "criterion_b_marginal_frac": round((with_b - plain) / plain, 4),
-            "roofline": {"bound": "tensor", "kernel": "forward (query tiles + value transpose + k_attn_fwd)",
+            "roofline": {"bound": "tensor", "kernel": "forward (k_prep + k_attn_fwd)",
                          "achieved": round(achieved, 2), "peak": bf16_s, "unit": "TFLOP/s",
                          "frac": round(achieved / bf16_s, 4), "peak_kind": peak_kind,
                          "algorithmic_flops_per_launch": flops},
@@ -505,6 +505,14 @@ def time_variants(args, call, stream, flush, torch, avtp, per_step):
     except Exception as e:  # a capture the runtime refuses: report it, keep the stream numbers
         out["graph"] = {"unavailable": f"{type(e).__name__}: {str(e)[:200]}"}
     return out
+
+
+def stage_launches(wl, criterion, lse=False, query_set="text"):
+    """Kernels of one avtp_prune call: k_prep, the scoring kernels (k_score_hvar; k_attn_pack,
+    k_attn_lse unless the LSE is supplied, k_attn_mass, k_attn_finalize; or k_narrow_logits and
+    k_narrow_mass), k_alloc_select (k_allocate and k_select for more than 32 images), k_compact."""
+    score = 1 if criterion == "hidden_variation" else 2 if query_set == "last" else 3 if lse else 4
+    return 2 + score + (2 if wl.layout.n_images > 32 else 1)
 
 
 def fa_lse(wl, q, k, torch):
@@ -574,10 +582,7 @@ def time_secondary(args, wl, L, kr, h_cur, pos, bf16, stream, flush, torch, avtp
             "latency_us": {"p50": round(step_ms[len(step_ms) // 2] * 1e3, 2),
                            "p90": round(step_ms[int(len(step_ms) * 0.9)] * 1e3, 2)},
             "steps_us": {k: round(v * 1e3, 2) for k, v in per_step.items()},
-            # k_prep, k_attn_pack, k_attn_lse (computed LSE only), k_attn_mass, k_attn_finalize,
-            # k_alloc_select, k_compact; the last-token set: k_prep, k_narrow_logits,
-            # k_narrow_mass, k_alloc_select, k_compact
-            "launches": K * ((7 if lse is None else 6) if query_set == "text" else 5)}
+            "launches": K * stage_launches(wl, "text_attention", lse is not None, query_set)}
 
 
 def forward_flops(wl):
@@ -688,7 +693,7 @@ def time_progressive(args, wl, L, h_cur, h_prior, pos, stream, flush, torch, avt
             "latency_us": {"p50": round(p50 * 1e3, 2), "p90": round(ms[int(len(ms) * 0.9)] * 1e3, 2)},
             "stage_roofline": {"bound": "hbm", "algorithmic_bytes": int(bytes_total), "bound_us": round(bound_us, 2),
                                "frac": round(bound_us / (p50 * 1e3), 4), "peak_gbs": hbm, "peak_kind": peak_kind},
-            "gpu_launches": K * (4 * stages + (stages - 1))}  # each boundary: one k_prep (it builds the spans)
+            "gpu_launches": K * (stage_launches(wl, "hidden_variation") * stages + (stages - 1))}  # each boundary: one k_prep (it builds the spans)
 
 
 def run_e2e(args, wl, crit, L, call, dev, stream, torch, avtp):
@@ -1254,18 +1259,19 @@ def run_timeline_attn(args):
         raise RuntimeError(f"device status (criterion-B timeline): {avtp.status_string(st)}")
     out = {"config": args.config, "unit": "SM cycles per step (median)"}
     for p in (1, 2):
-        def med(f):
+        def med(f, slots=()):  # slots: those not stamped at every step
             vals = []
             for t in stamps[p]:
                 n = int(np.count_nonzero(t[:, S["mma_issued"]]))  # steps the first CTA ran
-                vals += [f(t, j) for j in range(1, n)]
+                vals += [f(t, j) for j in range(1, n) if (t[j, list(slots)] != 0).all()]
             return round(float(np.median(vals)), 1) if vals else None
         out[f"pass{p}"] = {
             "steps_stamped": int(np.count_nonzero(stamps[p][-1][:, S["mma_issued"]])),
             "period": med(lambda t, j: t[j, S["mma_issued"]] - t[j - 1, S["mma_issued"]]),
             "mma_wait_for_operands": med(lambda t, j: t[j, S["mma_ready"]] - t[j, S["mma_step"]]),
             "mma_issue": med(lambda t, j: t[j, S["mma_issued"]] - t[j, S["mma_ready"]]),
-            "epilogue_hold": med(lambda t, j: t[j, S["acc_released"]] - t[j, S["acc_ready"]]),
+            "epilogue_hold": med(lambda t, j: t[j, S["acc_released"]] - t[j, S["acc_ready"]],
+                                 (S["acc_released"], S["acc_ready"])),
             "load_to_ready": med(lambda t, j: t[j, S["mma_ready"]] - t[j, S["load_issued"]])}
     return out
 

@@ -241,9 +241,10 @@ AVTP_API avtp_status_t avtp_forward_timeline(int64_t* out, int32_t max_blocks);
  * ran it, for the first max_steps (at most 64; the rest of out is left untouched) steps of
  * that CTA's run. Timeline build only
  * (AVTP_TIMELINE); the default build returns AVTP_ERR_UNSUPPORTED. out: host int64
- * [max_steps][6]: the key tile's load issued, the MMA thread at the step, its operands and
- * accumulators ready, its MMAs issued, the step's first accumulator ready for epilogue
- * warp 0, the step's last accumulator released by it. Synchronises the device. */
+ * [max_steps][6]: the key tile's load issued, the MMA thread of the block's first half at the
+ * step, its operands and accumulator ready, its MMAs issued, and on even steps that
+ * accumulator ready for epilogue warp 0 and released by it (odd steps belong to another
+ * warp: 0). Synchronises the device. */
 AVTP_API avtp_status_t avtp_score_timeline(int32_t pass, int64_t* out, int32_t max_steps);
 
 /* Step 2 (paper §3.3.3, App. A.2). From img_sums (device int64 [n_images]) writes

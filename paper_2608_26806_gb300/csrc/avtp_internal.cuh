@@ -178,8 +178,8 @@ constexpr int64_t kNarrowMaxLogitBytes = int64_t(1) << 30;
 // only when the batch has at most this many rows per KV group (decided from its text-token
 // bound). Measured on a request of four 640-token images and Qwen3-shaped heads (8 KV
 // groups of 4 heads, d = 128), score call event-timed: 29.3 us on the narrow path against
-// 34.4 us on tcgen05 at 4 rows per group (one text token), 33.4 against 34.4 at 8, and
-// the narrow path growing with the rows beyond (tcgen05 stays near 33 us up to 256 rows).
+// 31.7 us on tcgen05 at 4 rows per group (one text token), 33.8 against 31.7 at 8, and
+// the narrow path growing with the rows beyond (tcgen05 stays near 30 us up to 128 rows).
 constexpr int64_t kNarrowAutoRows = 4;
 struct NarrowPlan {
   int G;

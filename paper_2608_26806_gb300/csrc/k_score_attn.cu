@@ -103,8 +103,8 @@ __device__ __forceinline__ void bar_acc(int b, int t) {
 
 // Diagnostic timeline build (-DAVTP_TIMELINE): clock stamps of each pass's first CTA, per
 // step s of its run. Slots: 0 the key tile's load issued (TMA thread); 1 the MMA thread at
-// the step, 2 its operands and accumulators ready, 3 its MMAs issued and committed; 4 the
-// step's (first) accumulator ready for epilogue warp 0, 5 the step's (last) accumulator
+// the step, 2 its operands and accumulators ready, 3 its MMAs issued and committed (of the
+// block's first half); on even steps 4 that half's accumulator ready for epilogue warp 0, 5
 // released by it. Read with avtp_score_timeline().
 #ifdef AVTP_TIMELINE
 constexpr int kAttnTlSteps = 64;
