@@ -41,6 +41,8 @@
 // searches in the prefix arrays (AttnBlkInfo).
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "avtp_tc.cuh"
 
 namespace avtp {
@@ -231,7 +233,8 @@ __device__ __forceinline__ void p1_slice(uint32_t taddr, int pe, int lim, float 
 }
 
 // Pass 2: sum of exp2(c2 * z - lse2[c]) over the columns c >= c0 of a key's slice. `nlse`
-// holds -lse2. Chunks before c0 are not looked at; the one it falls into reads -inf there.
+// holds -lse2. Chunks before c0 are not looked at; in the one it falls into the exponents
+// before it read -inf, whatever logit or normaliser they came from.
 __device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, int c0, float c2) {
   // four partial sums (columns q mod 4), two per packed register
   float2 m01 = make_float2(0.f, 0.f), m23 = m01;
@@ -242,22 +245,27 @@ __device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, int
     tc::tmem_ld32_async(taddr + p * 32, r);
     const float4* l4 = reinterpret_cast<const float4*>(nlse + p * 32);
     tc::tmem_wait(r);
-    if (c0 > p * 32) {
+    auto sum = [&](auto edge) {
 #pragma unroll
-      for (int q = 0; q < 32; ++q) r[q] = (p * 32 + q >= c0) ? r[q] : 0xff800000u;
-    }
-#pragma unroll
-    for (int q4 = 0; q4 < 8; ++q4) {
-      const float4 lv = l4[q4];
-      const float2 a01 =
-          tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 0]), __uint_as_float(r[4 * q4 + 1])), cc,
-                    make_float2(lv.x, lv.y));
-      const float2 a23 =
-          tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3])), cc,
-                    make_float2(lv.z, lv.w));
-      m01 = tc::add2(m01, make_float2(tc::ex2(a01.x), tc::ex2(a01.y)));
-      m23 = tc::add2(m23, make_float2(tc::ex2(a23.x), tc::ex2(a23.y)));
-    }
+      for (int q4 = 0; q4 < 8; ++q4) {
+        const float4 lv = l4[q4];
+        float2 a01 = tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 0]), __uint_as_float(r[4 * q4 + 1])), cc,
+                               make_float2(lv.x, lv.y));
+        float2 a23 = tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3])), cc,
+                               make_float2(lv.z, lv.w));
+        if (decltype(edge)::value) {
+          const int c = p * 32 + 4 * q4;
+          a01.x = c + 0 >= c0 ? a01.x : -INFINITY;
+          a01.y = c + 1 >= c0 ? a01.y : -INFINITY;
+          a23.x = c + 2 >= c0 ? a23.x : -INFINITY;
+          a23.y = c + 3 >= c0 ? a23.y : -INFINITY;
+        }
+        m01 = tc::add2(m01, make_float2(tc::ex2(a01.x), tc::ex2(a01.y)));
+        m23 = tc::add2(m23, make_float2(tc::ex2(a23.x), tc::ex2(a23.y)));
+      }
+    };
+    if (c0 > p * 32) sum(std::true_type{});
+    else sum(std::false_type{});
   }
   return (m01.x + m01.y) + (m23.x + m23.y);
 }

@@ -68,6 +68,38 @@ def test_text_passes_moving_reference(heads, growth):
     _check(wl, scale=1.0)
 
 
+# ---------------------------------------------------------------- rows that a key is not scored by
+@pytest.mark.parametrize("heads", [(4, 2, 64), (8, 2, 128), (14, 2, 128)])
+@pytest.mark.parametrize("fill", [-np.inf, np.nan, np.inf])
+def test_normaliser_of_rows_before_an_image(heads, fill):
+    """A supplied normaliser counts for the images its query follows alone: one filled in behind
+    the first image only scores every image, and a query without one spoils the image before it
+    and not the image behind it."""
+    Hq, Hkv, d = heads
+    wl = synth.make_custom([[("t", 5), ("i", 40), ("t", 37), ("i", 130), ("t", 3), ("i", 9), ("t", 60)],
+                            [("t", 70), ("i", 140), ("t", 9)]], n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, hidden=64,
+                           seed=21, parts=("B",))
+    lay = wl.layout
+    lse = O.text_lse(lay, wl.q, wl.k, Hq, Hkv, wl.softmax_scale).astype(np.float32)
+    ref = O.score_text_attention(lay, wl.q, wl.k, Hq, Hkv, wl.softmax_scale, lse=lse.astype(np.float64))
+    second = int(lay.cu_seqlens[1])
+    lse[:, :5] = fill
+    lse[:, second:second + 70] = fill
+    L, q, k = dev_layout(lay), bf16_dev(wl.q), bf16_dev(wl.k)
+
+    def run(x):
+        scores, _ = avtp.score(L, "text_attention", q=q, k=k, softmax_scale=wl.softmax_scale, path="tensor",
+                               lse=torch.from_numpy(x).cuda())
+        return scores.cpu().numpy()
+
+    assert_scores_close(run(lse), ref, lay.visual_mask())
+    lse[:, 45 + 36] = np.nan  # the last query between the first two images
+    got, vis = run(lse), lay.visual_mask()
+    assert np.all(np.isnan(got[5:45]))
+    vis[5:45] = False
+    assert_scores_close(got, ref, vis)
+
+
 @pytest.mark.parametrize("bad", [{"cu_seqlens": [0, 900, 200]}, {"cu_seqlens": [0, -5, 200]},
                                  {"cu_seqlens": [7, 100, 200]}, {"img_start": [0, 180]}, {"img_len": [60, 0]}])
 def test_last_token_logits_beside_a_refused_layout(bad):
