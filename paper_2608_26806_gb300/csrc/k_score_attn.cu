@@ -16,10 +16,10 @@
 // Pass 2, k_attn_mass: the same with the roles exchanged: the tiles of 128 visual keys of
 // every image that one of the block's queries follows are the A operand, the block's halves
 // the B operand. A thread owns a key and sums exp2(z2 - lse2) over 128 rows, leaving out the
-// rows whose query precedes the key's image; lse2 comes from the pass-1 partials of the
-// block (merged when the walk enters it) or from the supplied LSE. The per-key sums of all
-// blocks and KV groups meet in a 64-bit fixed-point accumulator (integer atomics: the result
-// does not depend on their order).
+// rows whose query precedes the key's image and those of another request; lse2 comes from
+// the pass-1 partials of the block (merged when the walk enters it) or from the supplied
+// LSE. The per-key sums of all blocks and KV groups meet in a 64-bit fixed-point accumulator
+// (integer atomics: the result does not depend on their order).
 // k_attn_finalize turns the accumulator into scores and the fixed-point image sums.
 //
 // Both passes are persistent: the flat list of (KV group, block, key tile) is split into
@@ -232,40 +232,50 @@ __device__ __forceinline__ void p1_slice(uint32_t taddr, int pe, int lim, float 
   l += sum;
 }
 
-// Pass 2: sum of exp2(c2 * z - lse2[c]) over the columns c >= c0 of a key's slice. `nlse`
-// holds -lse2. Chunks before c0 are not looked at; in the one it falls into the exponents
-// before it read -inf, whatever logit or normaliser they came from.
-__device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, int c0, float c2) {
+// Pass 2: sum of exp2(c2 * z - lse2[c]) over the columns c0 <= c < c1 of a key's slice. `nlse`
+// holds -lse2. Chunks outside are not looked at; in those that c0 and c1 fall into the
+// exponents outside read -inf, whatever logit or normaliser they came from. A slice that is
+// live throughout has a loop of its own with a fixed end: with one loop for both, the score
+// call over eight requests (34423 tokens) took 150.0 us, so 146.5.
+__device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, int c0, int c1, float c2) {
   // four partial sums (columns q mod 4), two per packed register
   float2 m01 = make_float2(0.f, 0.f), m23 = m01;
   const float2 cc = make_float2(c2, c2);
-#pragma unroll 1
-  for (int p = c0 > 0 ? c0 >> 5 : 0; p < kChunks; ++p) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  auto chunk = [&](auto edge, int p, uint32_t live) {
     uint32_t r[32];
     tc::tmem_ld32_async(taddr + p * 32, r);
     const float4* l4 = reinterpret_cast<const float4*>(nlse + p * 32);
     tc::tmem_wait(r);
-    auto sum = [&](auto edge) {
 #pragma unroll
-      for (int q4 = 0; q4 < 8; ++q4) {
-        const float4 lv = l4[q4];
-        float2 a01 = tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 0]), __uint_as_float(r[4 * q4 + 1])), cc,
-                               make_float2(lv.x, lv.y));
-        float2 a23 = tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3])), cc,
-                               make_float2(lv.z, lv.w));
-        if (decltype(edge)::value) {
-          const int c = p * 32 + 4 * q4;
-          a01.x = c + 0 >= c0 ? a01.x : -INFINITY;
-          a01.y = c + 1 >= c0 ? a01.y : -INFINITY;
-          a23.x = c + 2 >= c0 ? a23.x : -INFINITY;
-          a23.y = c + 3 >= c0 ? a23.y : -INFINITY;
-        }
-        m01 = tc::add2(m01, make_float2(tc::ex2(a01.x), tc::ex2(a01.y)));
-        m23 = tc::add2(m23, make_float2(tc::ex2(a23.x), tc::ex2(a23.y)));
+    for (int q4 = 0; q4 < 8; ++q4) {
+      const float4 lv = l4[q4];
+      float2 a01 = tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 0]), __uint_as_float(r[4 * q4 + 1])), cc,
+                             make_float2(lv.x, lv.y));
+      float2 a23 = tc::ffma2(make_float2(__uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3])), cc,
+                             make_float2(lv.z, lv.w));
+      if (decltype(edge)::value) {
+        a01.x = (live >> (4 * q4 + 0)) & 1u ? a01.x : -INFINITY;
+        a01.y = (live >> (4 * q4 + 1)) & 1u ? a01.y : -INFINITY;
+        a23.x = (live >> (4 * q4 + 2)) & 1u ? a23.x : -INFINITY;
+        a23.y = (live >> (4 * q4 + 3)) & 1u ? a23.y : -INFINITY;
       }
-    };
-    if (c0 > p * 32) sum(std::true_type{});
-    else sum(std::false_type{});
+      m01 = tc::add2(m01, make_float2(tc::ex2(a01.x), tc::ex2(a01.y)));
+      m23 = tc::add2(m23, make_float2(tc::ex2(a23.x), tc::ex2(a23.y)));
+    }
+  };
+  if (c0 <= 0 && c1 >= kHalf) {
+#pragma unroll 1
+    for (int p = 0; p < kChunks; ++p) chunk(std::false_type{}, p, kAll);
+  } else {
+    const int pe = min(kChunks, (c1 + 31) >> 5);
+#pragma unroll 1
+    for (int p = c0 > 0 ? c0 >> 5 : 0; p < pe; ++p) {
+      const int lo = c0 - p * 32, hi = c1 - p * 32;
+      const uint32_t live = (lo > 0 ? kAll << lo : kAll) & (hi < 32 ? ~(kAll << hi) : kAll);
+      if (live != kAll) chunk(std::true_type{}, p, live);
+      else chunk(std::false_type{}, p, kAll);
+    }
   }
   return (m01.x + m01.y) + (m23.x + m23.y);
 }
@@ -617,8 +627,8 @@ k_attn_mass(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
             lse_own = M + log2f(L);
           }
         }
-        // rows past the request's carry -inf, which makes their terms vanish; thread etid's
-        // row is one that its own accumulator's threads read
+        // thread etid's row is one that its own accumulator's threads read; rows past the
+        // request's (another request's, or none) are left out by p2_slice
         par ^= 1;
         s_lse[t][par][etid] = -lse_own;
         bar_acc(t, half);
@@ -635,7 +645,7 @@ k_attn_mass(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
       // does this warp's row half hold a visible row? (uniform over its group)
       const bool any = c0 < (half + 1) * kHalf && c1 > half * kHalf;
       float mass = 0.f;
-      if (ok && any) mass = p2_slice(taddr, &s_lse[t][par][half * kHalf], c0 - half * kHalf, c2);
+      if (ok && any) mass = p2_slice(taddr, &s_lse[t][par][half * kHalf], c0 - half * kHalf, c1 - half * kHalf, c2);
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&sy.acc_empty[t][half]);

@@ -2,6 +2,8 @@
 key tiles of 128 and their remainders, row blocks of 256 and their halves, runs of a CTA that
 cross blocks, first visible rows inside a 32-row chunk, and a softmax reference that moves.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -98,6 +100,60 @@ def test_normaliser_of_rows_before_an_image(heads, fill):
     assert np.all(np.isnan(got[5:45]))
     vis[5:45] = False
     assert_scores_close(got, ref, vis)
+
+
+@pytest.mark.parametrize("heads", [(4, 2, 64), (3, 1, 128), (8, 2, 128)])
+@pytest.mark.parametrize("n", [1, 15, 16, 31, 32, 33, 64, 65, 127, 128, 129])
+@pytest.mark.parametrize("how", ["own", "lse", "forward"])
+def test_scores_ignore_what_other_requests_hold(heads, n, how):
+    """A request's last row block reads rows of the next request: infinities and NaN there stay there."""
+    Hq, Hkv, d = heads
+    wl = synth.make_custom([[("i", 3), ("t", 2)], [("i", 70), ("t", 1), ("i", 30), ("t", n)], [("i", 40), ("t", 300)]],
+                           n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, hidden=64, seed=100 + n, parts=("B", "V"))
+    lay, scale = wl.layout, wl.softmax_scale
+    a, b = int(lay.cu_seqlens[1]), int(lay.cu_seqlens[2])
+    lse = O.text_lse(lay, wl.q, wl.k, Hq, Hkv, scale).astype(np.float32)
+    ref = O.score_text_attention(lay, wl.q, wl.k, Hq, Hkv, scale)
+    L, q, k = dev_layout(lay), bf16_dev(wl.q), bf16_dev(wl.k)
+    lse = torch.from_numpy(lse).cuda()
+    for t, x in ((q, float("nan")), (k, float("inf"))):
+        t[:a], t[b:] = x, x
+    lse[:, :a], lse[:, b:] = float("nan"), float("nan")
+    if how == "forward":
+        _, _, scores, sums = avtp.attn_forward(L, q=q, k=k, v=bf16_dev(wl.v), softmax_scale=scale, path="tensor")
+    else:
+        scores, sums = avtp.score(L, "text_attention", q=q, k=k, softmax_scale=scale, path="tensor",
+                                  lse=lse if how == "lse" else None)
+    got = scores.cpu().numpy()
+    mine = lay.visual_mask() & (np.arange(lay.n_tokens) >= a) & (np.arange(lay.n_tokens) < b)
+    assert_scores_close(got, ref, mine)
+    assert np.array_equal(sums.cpu().numpy()[1:3], O.image_sums(lay, got)[1:3])
+
+
+@pytest.mark.parametrize("supplied", [False, True])
+def test_scores_with_a_loose_text_bound(supplied):
+    """Rows between the batch's text and a looser bound on it are workspace nothing has written."""
+    Hq, Hkv, d = 8, 2, 128
+    wl = synth.make_custom([[("i", 140), ("t", 30)], [("t", 2), ("i", 70), ("t", 41)]], n_q_heads=Hq, n_kv_heads=Hkv,
+                           head_dim=d, hidden=64, seed=8, parts=("B",))
+    lay, scale = wl.layout, wl.softmax_scale
+    lse = O.text_lse(lay, wl.q, wl.k, Hq, Hkv, scale).astype(np.float32)
+    ref = O.score_text_attention(lay, wl.q, wl.k, Hq, Hkv, scale)
+    L, q, k, lse = dev_layout(lay), bf16_dev(wl.q), bf16_dev(wl.k), torch.from_numpy(lse).cuda()
+    for bound in (0, 100, lay.n_tokens):
+        sa = avtp._score_args("text_attention", q=q, k=k, softmax_scale=scale, lse=lse if supplied else None,
+                              max_text_tokens=bound, path="tensor")
+        cl, size = L.c(), ctypes.c_size_t()
+        lib = avtp.load()
+        assert lib.avtp_workspace_size(ctypes.byref(cl), ctypes.byref(sa), ctypes.byref(size)) == avtp.OK
+        ws = torch.full((size.value,), 0xFF, dtype=torch.uint8, device="cuda")
+        scores = torch.zeros(lay.n_tokens, device="cuda")
+        sums = torch.zeros(lay.n_images, dtype=torch.int64, device="cuda")
+        assert lib.avtp_score(ctypes.byref(cl), ctypes.byref(sa), scores.data_ptr(), sums.data_ptr(), ws.data_ptr(),
+                              size.value, avtp._stream(None)) == avtp.OK
+        torch.cuda.synchronize()
+        assert avtp.read_device_status(ws) == avtp.OK
+        assert_scores_close(scores.cpu().numpy(), ref, lay.visual_mask())
 
 
 @pytest.mark.parametrize("bad", [{"cu_seqlens": [0, 900, 200]}, {"cu_seqlens": [0, -5, 200]},
