@@ -15,6 +15,7 @@ namespace {
 
 constexpr int kMaxWarpsPerCta = 4;
 constexpr size_t kSmemBudget = 200 * 1024;
+static_assert(warp_alloc_smem_bytes(kMaxImagesPerRequest) <= kSmemBudget, "one warp's scratch fits at any size");
 
 __global__ void __launch_bounds__(kMaxWarpsPerCta * 32, 1)
 k_allocate(const int32_t* __restrict__ img_cu, const int32_t* __restrict__ img_len,
@@ -101,11 +102,14 @@ cudaError_t launch_allocate(const avtp_layout_t& L, const int64_t* img_sums, con
   int wpc = static_cast<int>(kSmemBudget / per_warp);
   wpc = wpc < 1 ? 1 : (wpc > kMaxWarpsPerCta ? kMaxWarpsPerCta : wpc);
   const size_t smem = wpc * per_warp;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_allocate, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-  }
+  // the attribute belongs to the device and not to the call, and other threads may launch: set
+  // once, to the most that any call asks for
+  static PerDevice attrs;
+  const cudaError_t ae = once_per_device(attrs, [](int, int*) {
+    return cudaFuncSetAttribute(k_allocate, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(kSmemBudget));
+  });
+  if (ae != cudaSuccess) return ae;
   const int grid = (L.n_requests + wpc - 1) / wpc;
   return launch_kernel(k_allocate, dim3(grid), dim3(32 * wpc), smem, s, /*pdl=*/true, L.img_cu, L.img_len, img_sums,
                        aa.keep_ratio, aa.alpha, aa.r_min, aa.r_max, aa.relative, ws_at<int32_t>(ws, p.vis_cu),

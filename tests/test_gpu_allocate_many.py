@@ -4,6 +4,9 @@ the oracle, in avtp_allocate and in the fused stage: images per request about 32
 remainders at the largest-remainder cut. And batches of about as many requests as a warp has
 lanes, some without images, where each image finds its request.
 """
+import ctypes
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -104,3 +107,44 @@ def test_fused_stage_many_requests(n_req, empty):
     assert np.array_equal(out.kept_idx.cpu().numpy(), ref["kept_idx"])
     kept = torch.from_numpy(ref["kept_idx"].astype(np.int64)).cuda()
     assert torch.equal(out.outputs["hidden"].view(torch.int16), h_cur[kept].view(torch.int16))
+
+
+def test_two_threads_of_different_sizes():
+    """Two host threads, each with a stream of its own, allocate for batches whose rule takes
+    different amounts of shared memory (an image's worth for every image of the batch, four
+    warps a CTA); no call of either is refused, and both stay right."""
+    lib = avtp.load()
+    jobs = []
+    for n_req in (64, 250):
+        rng = np.random.default_rng(n_req)
+        lay = synth.Layout.from_segments([[("t", 2)] + [("i", int(n)) for n in rng.integers(1, 300, size=4)]
+                                          for _ in range(n_req)])
+        S = _sums(rng, lay.img_len.astype(np.int64), "mild")
+        kr = np.full(n_req, 0.5, dtype=np.float32)
+        L = dev_layout(lay)
+        t = [torch.from_numpy(S).cuda(), torch.from_numpy(kr).cuda(),
+             torch.empty(lay.n_images, dtype=torch.int32, device="cuda"),
+             torch.empty(n_req + 1, dtype=torch.int32, device="cuda"), avtp.new_workspace(avtp.workspace_size(L))]
+        structs = (L.c(), avtp._alloc_args(t[1]))
+        stream = torch.cuda.Stream()
+        args = (ctypes.byref(structs[0]), t[0].data_ptr(), ctypes.byref(structs[1]), t[2].data_ptr(), t[3].data_ptr(),
+                t[4].data_ptr(), t[4].numel(), stream.cuda_stream)
+        jobs.append(dict(args=args, budgets=t[2], ws=t[4], keep=(L, t, structs, stream), codes=[],
+                         ref=O.allocate(lay, S, kr, 1.0, 0.05, 0.95, False)["budgets"]))
+    torch.cuda.synchronize()
+    gate = threading.Barrier(2)
+
+    def work(job):
+        gate.wait()
+        job["codes"] = [lib.avtp_allocate(*job["args"]) for _ in range(20000)]
+
+    threads = [threading.Thread(target=work, args=(job,)) for job in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for job in jobs:
+        assert job["codes"].count(avtp.OK) == len(job["codes"])
+        assert avtp.read_device_status(job["ws"]) == avtp.OK
+        assert np.array_equal(job["budgets"].cpu().numpy(), job["ref"])
