@@ -342,9 +342,10 @@ static __device__ __noinline__ int exact_multi(const WarpAllocSmem& sm, int m, b
 // All 32 lanes call with identical scalars. sm.S[j] = S_j and sm.n[j] = n_j for j < m on
 // entry; the budgets are left in sm.K. Returns AVTP_OK, AVTP_ERR_DEVICE_INPUT for a sum
 // beyond n_j * 2^42, or AVTP_ERR_RANGE if the rounding loop did not converge (never
-// expected).
+// expected). dry: a warm-up on made-up sums, which ends where the register form does: what
+// lies behind it takes longer than most scorings (see k_allocate).
 static __device__ __noinline__ int warp_allocate(const WarpAllocSmem& sm, int m, int64_t B, int32_t N, float r_base_f,
-                                                 float alpha_f, float r_min_f, float r_max_f, int relative) {
+                                                 float alpha_f, float r_min_f, float r_max_f, int relative, bool dry) {
   const int lane = threadIdx.x & 31;
   const int64_t Rmin = ratio_grid(r_min_f), Rmax = ratio_grid(r_max_f);
   // ---- ratios on the grid
@@ -368,7 +369,7 @@ static __device__ __noinline__ int warp_allocate(const WarpAllocSmem& sm, int m,
   };
   if (m <= kMultiImages) {
     const int err = multi(true, 0);
-    if (err != kExactFallback) return err;
+    if (err != kExactFallback || dry) return err;
   }
   const int64_t avg = grid_mean(T, recip62(N));
   const int64_t inv_avg = (relative && avg != 0) ? recip62(avg > 0 ? avg : -avg) : 0;
@@ -716,7 +717,8 @@ static __device__ __noinline__ int general_stage32(const WarpAllocSmem& sm, int 
 // caller's state on the stack.
 __device__ __forceinline__ int warp_allocate32(const WarpAllocSmem& sm, int m, int64_t S, int32_t n, int64_t inv_n,
                                                    int64_t B, int32_t N, int64_t inv_N, const RatioRule& rule,
-                                                   float alpha_f, float r_min_f, float r_max_f, int32_t* k_out) {
+                                                   float alpha_f, float r_min_f, float r_max_f, int32_t* k_out,
+                                                   bool dry = false) {
   const int lane = threadIdx.x & 31;
   const bool has = lane < m;
   const int64_t lim = static_cast<int64_t>(n) << kSumMagnitudeBits;
@@ -739,7 +741,7 @@ __device__ __forceinline__ int warp_allocate32(const WarpAllocSmem& sm, int m, i
     const int64_t g = R + lam;
     cls = g <= Rmin ? kClsLow : (g >= Rmax ? kClsHigh : kClsFree);
   }
-  if (err == kExactFallback)
+  if (err == kExactFallback && !dry)
     err = general_stage32(sm, m, S, n, R, B, N, T, rule, alpha_f, r_min_f, r_max_f, lam, Rmin, Rmax, &K);
   *k_out = K;
   return err;
