@@ -199,10 +199,12 @@ int device_sm_count() {
 // SMs the scoring kernel leaves to the selection kernel, at most.
 constexpr int kMaxReserveSms = 32;
 
-int prune_reserve_sms(const avtp_layout_t& L) {
-  if (L.n_images > kFusedImages) return 1;  // k_allocate's
+int prune_reserve_sms(const avtp_layout_t& L, int64_t hidden) {
+  // k_allocate's; without a warm-up it gains on small batches alone (16 requests of 3 images,
+  // hidden 256: of 65 tokens 17.1 us with an SM left free and 18.6 without, of 1000 54.0 and 52.8)
+  if (L.n_images > kFusedImages) return prune_warm_ctas(L, hidden) > 0 || L.n_tokens <= 16384 ? 1 : 0;
   if (L.n_tokens > 32768 || L.n_images < 1) return 0;
-  const int64_t ctas = prune_warm_ctas(L);
+  const int64_t ctas = prune_warm_ctas(L, hidden);
   // one SM per selection CTA (its registers fill most of an SM; two on one SM slowed each
   // other's budget rule) and one for the validation kernel, which runs when the scoring
   // kernel starts: at most kMaxReserveSms, the CTAs beyond start when the scoring
@@ -210,8 +212,12 @@ int prune_reserve_sms(const avtp_layout_t& L) {
   return static_cast<int>(ctas + 1 < kMaxReserveSms ? ctas + 1 : kMaxReserveSms);
 }
 
-int prune_warm_ctas(const avtp_layout_t& L) {
-  if (L.n_images > kFusedImages) return 1;  // k_allocate's
+int prune_warm_ctas(const avtp_layout_t& L, int64_t hidden) {
+  if (L.n_images > kFusedImages) {
+    // k_allocate's first, the one that has an SM left free
+    const bool many = L.n_images > 32 * static_cast<int64_t>(L.n_requests);
+    return many || L.n_tokens >= kWarmScoreBytes / (4 * hidden) ? 1 : 0;
+  }
   if (L.n_tokens > 32768 || L.n_images < 1) return 0;
   const int64_t ctas = static_cast<int64_t>(L.n_images) + L.n_requests;
   return ctas <= kMaxWarmCtas ? static_cast<int>(ctas) : 0;
@@ -413,10 +419,11 @@ avtp_status_t avtp_prune(const avtp_layout_t* layout, const avtp_score_args_t* s
   }
   if ((st = from_cuda(launch_prep(pa, workspace, p, s))) != AVTP_OK) return st;
   if ((st = record(step_events, 1, s)) != AVTP_OK) return st;
-  const int reserve = score_args->criterion == AVTP_CRIT_HIDDEN_VARIATION ? prune_reserve_sms(*layout) : 0;
+  const bool hidden_criterion = score_args->criterion == AVTP_CRIT_HIDDEN_VARIATION;
+  const int reserve = hidden_criterion ? prune_reserve_sms(*layout, score_args->hidden) : 0;
   if ((st = score_impl(layout, score_args, sc, sums, workspace, p, s, reserve)) != AVTP_OK) return st;
   if ((st = record(step_events, 2, s)) != AVTP_OK) return st;
-  const int warm = score_args->criterion == AVTP_CRIT_HIDDEN_VARIATION ? prune_warm_ctas(*layout) : 0;
+  const int warm = hidden_criterion ? prune_warm_ctas(*layout, score_args->hidden) : 0;
   if ((st = from_cuda(launch_alloc_select(*layout, sums, *alloc_args, budgets, sc, out_cu_seqlens, kept_idx, n_kept,
                                           workspace, p, s, warm))) != AVTP_OK)
     return st;

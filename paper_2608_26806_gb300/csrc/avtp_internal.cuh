@@ -358,7 +358,8 @@ cudaError_t launch_attn_finalize(const avtp_layout_t& L, const avtp_score_args_t
                                  int64_t* img_sums, void* ws, const WsPlan& p, const AttnPlan& plan, cudaStream_t s);
 
 cudaError_t launch_allocate(const avtp_layout_t& L, const int64_t* img_sums, const avtp_alloc_args_t& aa,
-                            int32_t* budgets, void* ws, const WsPlan& p, cudaStream_t s, bool warm = false);  // warm: see k_allocate.cu
+                            int32_t* budgets, void* ws, const WsPlan& p, cudaStream_t s,
+                            int warm_ctas = 0);  // warm_ctas: see k_allocate.cu
 
 cudaError_t launch_select(const avtp_layout_t& L, const float* scores, const int32_t* budgets,
                           const int32_t* out_cu_seqlens, int32_t* kept_idx, int64_t n_kept, void* ws,
@@ -383,11 +384,18 @@ cudaError_t launch_alloc_select(const avtp_layout_t& L, const int64_t* img_sums,
 // their instruction caches (prune_warm_ctas(L) of them run the code once on made-up data
 // first); 0 otherwise. Right after the scoring stream has swept L2 a cold run of the
 // budget rule and the selection takes several times longer. On large batches the
-// scoring time would grow instead. Batches of more images leave one SM, to k_allocate.
+// scoring time would grow instead. Batches of more images leave one SM to k_allocate, whose
+// first CTA (up to four requests) warms up on it; with at most 32 images a request on average only
+// where the scoring reads kWarmScoreBytes or more: a shorter one ends before the warm-up does.
+// Stage, warmed up and not: two requests of 32 images of 16 tokens, hidden 256, 26.9 / 15.2 us,
+// eight of 24 of 16, hidden 4096 (41 MB), 27.0 / 21.3, sixteen of 24 of 16, 4096 (82 MB), 27.2 /
+// 27.2, two of 32 of 256, 4096 (270 MB), 56.3 / 57.9. Larger requests' rule gains at any length:
+// 64 images of 256 tokens, hidden 64 (4 MB), 31.3 / 33.6. Every CTA of eight requests of 16
+// images of 16 tokens warming up took 27.9 us, its first alone 26.9, none 16.6.
 constexpr int kMaxWarmCtas = 96;
-int prune_reserve_sms(const avtp_layout_t& L);
-int prune_warm_ctas(const avtp_layout_t& L);
-
+constexpr int64_t kWarmScoreBytes = 56 << 20;
+int prune_reserve_sms(const avtp_layout_t& L, int64_t hidden);
+int prune_warm_ctas(const avtp_layout_t& L, int64_t hidden);
 
 cudaError_t launch_compact(const int32_t* kept_idx, int64_t n_kept, int64_t n_tokens, const avtp_rows_t* sets,
                            int n_sets, void* ws, const WsPlan& p, cudaStream_t s);

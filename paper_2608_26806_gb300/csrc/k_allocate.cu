@@ -4,10 +4,10 @@
 // four or eight images a lane up to 256, shared memory beyond. avtp_prune of more than kFusedImages images
 // runs it between the scores and k_select.
 // Latency and instruction fetches bound it: right behind the scoring stream, which sweeps L2,
-// a cold run of the rule takes 15-25 us, most of it fetching code. With warm the kernel, which
-// starts beside the scoring on an SM left free for it, runs the rule once on made-up sums
-// before it waits: the stage of 64 images of one request 72 -> 67 us, of eight requests of five
-// images 68 -> 61 us.
+// a cold run of the rule takes 15-25 us, most of it fetching code. The first warm_ctas CTAs,
+// which start beside the scoring on an SM left free for them, run the rule once on made-up sums
+// before they wait: the stage of 64 images of one request 72 -> 67 us, of eight requests of five
+// images 68 -> 61 us. The CTAs that start behind the scoring have nothing to hide it behind.
 #include "avtp_alloc.cuh"
 
 namespace avtp {
@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32, 1)
 k_allocate(const int32_t* __restrict__ img_cu, const int32_t* __restrict__ img_len,
            const int64_t* __restrict__ img_sums, const float* __restrict__ keep_ratio, float alpha, float r_min,
            float r_max, int relative, const int32_t* __restrict__ vis_cu, int32_t* req_budget,
-           int32_t* __restrict__ budgets, int R, int NI, int m_cap, int warm, DevStatus* st) {
+           int32_t* __restrict__ budgets, int R, int NI, int m_cap, int warm_ctas, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -43,7 +43,7 @@ k_allocate(const int32_t* __restrict__ img_cu, const int32_t* __restrict__ img_l
   int err = AVTP_OK;
   // one copy of the code for the warm-up and the real run
 #pragma unroll 1
-  for (int pass = warm && m <= kMultiImages ? 0 : 1; pass < 2; ++pass) {
+  for (int pass = static_cast<int>(blockIdx.x) < warm_ctas && m <= kMultiImages ? 0 : 1; pass < 2; ++pass) {
     int64_t S = 0, B;
     int32_t N;
     if (pass == 1) {
@@ -100,7 +100,7 @@ k_allocate(const int32_t* __restrict__ img_cu, const int32_t* __restrict__ img_l
 }  // namespace
 
 cudaError_t launch_allocate(const avtp_layout_t& L, const int64_t* img_sums, const avtp_alloc_args_t& aa,
-                            int32_t* budgets, void* ws, const WsPlan& p, cudaStream_t s, bool warm) {
+                            int32_t* budgets, void* ws, const WsPlan& p, cudaStream_t s, int warm_ctas) {
   if (L.n_images == 0) return cudaSuccess;
   const int m_cap = L.n_images < kMaxImagesPerRequest ? L.n_images : kMaxImagesPerRequest;
   const size_t per_warp = warp_alloc_smem_bytes(m_cap);
@@ -118,7 +118,7 @@ cudaError_t launch_allocate(const avtp_layout_t& L, const int64_t* img_sums, con
   const int grid = (L.n_requests + wpc - 1) / wpc;
   return launch_kernel(k_allocate, dim3(grid), dim3(32 * wpc), smem, s, /*pdl=*/true, L.img_cu, L.img_len, img_sums,
                        aa.keep_ratio, aa.alpha, aa.r_min, aa.r_max, aa.relative, ws_at<int32_t>(ws, p.vis_cu),
-                       ws_at<int32_t>(ws, p.req_budget), budgets, L.n_requests, L.n_images, m_cap, warm ? 1 : 0,
+                       ws_at<int32_t>(ws, p.req_budget), budgets, L.n_requests, L.n_images, m_cap, warm_ctas,
                        ws_at<DevStatus>(ws, p.status));
 }
 

@@ -665,7 +665,7 @@ cudaError_t launch_alloc_select(const avtp_layout_t& L, const int64_t* img_sums,
                                 int32_t* kept_idx, int64_t n_kept, void* ws, const WsPlan& p, cudaStream_t s,
                                 int warm_ctas) {
   if (L.n_images > kFusedImages) {
-    const cudaError_t e = launch_allocate(L, img_sums, aa, budgets, ws, p, s, /*warm=*/warm_ctas > 0);
+    const cudaError_t e = launch_allocate(L, img_sums, aa, budgets, ws, p, s, warm_ctas);
     if (e != cudaSuccess) return e;
     return launch_select(L, scores, budgets, out_cu_seqlens, kept_idx, n_kept, ws, p, s, /*after_allocate=*/true);
   }
