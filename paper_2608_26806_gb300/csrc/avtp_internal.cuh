@@ -31,7 +31,17 @@ constexpr int kAttnTileM = 128;          // keys of a tile, rows of a product
 constexpr int kAttnBlockRows = 256;      // rows per block (both passes)
 constexpr int kAttnMaxChunks = 64;       // pass-1 partial (max, sum) slots per row at most
 constexpr int kAttnMaxGroupHeads = 128;  // Hq / Hkv at most
-constexpr int kAttnMassFracBits = 40;    // fixed point of the per-key probability mass
+constexpr int kAttnMassFracBits = 40;    // fixed point of the per-key probability mass, at most (attn_mass_frac_bits)
+// A block's mass of a key, at most: one per row, and room for a supplied normaliser's rounding
+// (a larger one is flagged, see k_score_attn.cu).
+constexpr int kAttnBlockMassBits = 9;
+static_assert((1 << kAttnBlockMassBits) > kAttnBlockRows, "a block's mass");
+// The fraction bits that keep the sum over `adds` (KV group, block)s of one request below the
+// accumulator's top bit: 40 for fewer than 2^14, which are 2^22 (text query, head)s.
+__device__ __forceinline__ int attn_mass_frac_bits(int64_t adds) {
+  const int len = 64 - __clzll(adds);  // adds < 2^len; fewer than 2^48: rows are 32-bit numbers
+  return min(kAttnMassFracBits, 63 - kAttnBlockMassBits - len);
+}
 
 // What the two passes need of a row block, laid out by the validation kernel (as two int4)
 // so that a walk over blocks takes one load where the prefix arrays would take a search.
@@ -145,7 +155,7 @@ struct WsPlan {
   size_t p2t_cu;      // int32 [n_blocks_max + 1]: pass-2 key tiles per row block
   size_t ktile_cu;    // int32 [n_img + 1]: key tiles per image
   size_t ktile_img;   // int32 [n_ktiles_max]: image of every key tile
-  size_t meta;        // int32 [8]: F1, C1, F2, C2 (flat pass lengths per KV group, steps per CTA), row blocks
+  size_t meta;        // int32 [8]: F1, C1, F2, C2 (flat pass lengths per KV group, steps per CTA), row blocks, mass bits
   size_t blk_info;    // AttnBlkInfo [n_blocks_max]
   size_t tile_info;   // int4 [n_ktiles_max]: see AttnBlkInfo
   size_t cta_start;   // int4 [2][grid]: see AttnBlkInfo

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kPrepThreads)
 k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t* req_budget, int32_t* text_idx,
        int32_t* text_cu, int32_t* blk_cu, int32_t* p1s_cu, int32_t* p2t_cu, int32_t* ktile_cu, int32_t* ktile_img,
        int32_t* meta, int4* blk_info, int4* tile_info, int4* cta_start, int32_t* g_scratch) {
-  __shared__ int s_err, s_detail, s_max_steps;
+  __shared__ int s_err, s_detail, s_max_steps, s_max_blocks;
   __shared__ int32_t s_warp[32];
   __shared__ int32_t s_stage[kStageInts];
   __shared__ int32_t s_list[kText ? 2 : 1][kText ? kStageBlocks + 1 : 1];
@@ -244,7 +244,7 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
       block_exclusive_scan<int32_t>(NB, p2_tiles, p2t_cu, s_warp);
       // Pass 1 of block b: steps of kAttnTileM keys from the request's first token to its
       // last query (none when pass 2 has nothing for the block).
-      if (tid == 0) s_max_steps = 0;
+      if (tid == 0) s_max_steps = s_max_blocks = 0;
       __syncthreads();
       auto p1_steps = [&](int b) {
         if (p2t_cu[b + 1] == p2t_cu[b]) return 0;
@@ -254,6 +254,7 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
         const int keys = text_idx[(R1 - 1) / G] - cu[r] + 1;
         const int steps = (keys + kAttnTileM - 1) / kAttnTileM;
         atomicMax(&s_max_steps, steps);
+        atomicMax(&s_max_blocks, b - blk_cu[r] + 1);
         return steps;
       };
       block_exclusive_scan<int32_t>(NB, p1_steps, p1s_cu, s_warp);
@@ -284,6 +285,7 @@ k_prep(PrepArgs a, DevStatus* st, int32_t* g_vis_cu, int32_t* g_img_req, int32_t
           meta[3] = static_cast<int32_t>(C2);
           meta[4] = NB;
         }
+        if (tid == 32) meta[5] = attn_mass_frac_bits(static_cast<int64_t>(a.attn.Hkv) * s_max_blocks);
         for (int64_t c = tid; c < 2 * grid; c += blockDim.x) {
           const int pass = c >= grid ? 1 : 0;
           const int64_t F = pass ? F2 : F1, C = pass ? C2 : C1;

@@ -59,9 +59,9 @@ constexpr uint32_t kTmemCols = 512;  // four accumulators of 128 columns
 constexpr int kStages = 4;            // key tiles in flight
 constexpr int kMassWindow = 12;       // steps of an epilogue group whose key masses are held in shared memory between flushes
 constexpr float kLog2e = 1.4426950408889634f;
-// Flag of a key whose mass is not a finite number in [0, 256] (non-finite inputs). The
-// sum of its finite contributions stays below 2^62: at most 256 * 2^40 per (KV group,
-// block), fewer than 2^14 of them.
+// Flag of a key whose mass in some block is not a number in [0, 2^kAttnBlockMassBits]
+// (non-finite inputs, or a supplied normaliser far below the row's own). The sum of its finite
+// contributions stays below this bit (attn_mass_frac_bits).
 constexpr unsigned long long kMassNotFinite = 1ull << 63;
 
 static_assert(kBlk == 2 * kM, "a block is two products of 128 rows");
@@ -85,10 +85,10 @@ struct AttnArgs {
   const int4* blk_info;          // the validation kernel's tables, see AttnBlkInfo
   const int4* tile_info;
   const int4* cta_start;
-  const int32_t* meta;           // F1, C1, F2, C2, NB
+  const int32_t* meta;           // F1, C1, F2, C2, NB, fraction bits of the mass
   const float* lse_rows;         // [Hkv, rows] (supplied LSE) or nullptr
   float2* p1_part;               // [Hkv * NB][256 rows][kAttnMaxChunks]
-  unsigned long long* mass;      // [key tile][128] fixed point, 2^-kAttnMassFracBits
+  unsigned long long* mass;      // [key tile][128] fixed point, 2^-meta[5]
   int64_t rows;
   int G;
   float c2;                      // softmax_scale * log2(e)
@@ -279,6 +279,9 @@ __device__ __forceinline__ float p2_slice(uint32_t taddr, const float* nlse, int
   }
   return (m01.x + m01.y) + (m23.x + m23.y);
 }
+
+// 2^e, -126 <= e <= 127.
+__device__ __forceinline__ float pow2(int e) { return __int_as_float((127 + e) << 23); }
 
 __device__ __forceinline__ void setup_sync(Sync& sy, int warp) {
   if (threadIdx.x == 0) {
@@ -659,13 +662,14 @@ k_attn_mass(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CU
         // flush: one fixed-point integer add per (step, key), both column halves summed
         // in fp32 first (integer adds: the result does not depend on their order)
         bar_set(t);
+        const float mass_scale = pow2(a.meta[5]);
         for (int e = etid; e < w * kM; e += kSetThreads) {
           const int ws = e / kM, k = e % kM;
           if (k < s_nk[t][ws]) {
             const float m = s_mass[t][ws][0][k] + s_mass[t][ws][1][k];
             unsigned long long* dst = a.mass + static_cast<int64_t>(s_tile[t][ws]) * kM + k;
-            if (m <= 512.f) {  // at most one per row of the block
-              atomicAdd(dst, static_cast<unsigned long long>(__float2ll_rn(m * static_cast<float>(1ull << kAttnMassFracBits))));
+            if (m <= static_cast<float>(1 << kAttnBlockMassBits)) {
+              atomicAdd(dst, static_cast<unsigned long long>(__float2ll_rn(m * mass_scale)));
             } else {
               atomicOr(dst, kMassNotFinite);  // NaN or inf inputs: the key scores NaN (bit 63; finite adds never reach it)
             }
@@ -716,12 +720,12 @@ k_attn_pack(const __nv_bfloat16* __restrict__ q, int64_t q_stride, int Hq, int G
 }
 
 // ---------------------------------------------------------------- finalize
-// One CTA per key tile (128 keys of one image): s_t = mass_t * 2^-40 / (Hq * |Q_r|), and
+// One CTA per key tile (128 keys of one image): s_t = mass_t * 2^-bits / (Hq * |Q_r|), and
 // the tile's fixed-point score sum added to its image's sum with one atomic.
 __global__ void __launch_bounds__(kM)
 k_attn_finalize(const unsigned long long* __restrict__ mass, const int32_t* __restrict__ ktile_cu,
                 const int32_t* __restrict__ ktile_img, const int4* __restrict__ tile_info, int Hq,
-                const int32_t* __restrict__ text_cu, int NI, float* __restrict__ scores,
+                const int32_t* __restrict__ text_cu, const int32_t* __restrict__ meta, int NI, float* __restrict__ scores,
                 int64_t* __restrict__ img_sums, const DevStatus* st) {
   __shared__ long long s_part[kM / 32];
   pdl_wait();
@@ -732,6 +736,7 @@ k_attn_finalize(const unsigned long long* __restrict__ mass, const int32_t* __re
     const int4 info = tile_info[tile];
     const unsigned long long m = mass[static_cast<int64_t>(tile) * kM + threadIdx.x];
     const int nq = text_cu[info.w + 1] - text_cu[info.w];  // the request's queries
+    const float unit = pow2(-meta[5]);
     long long fx = 0;
     if (static_cast<int>(threadIdx.x) < info.y) {
       float s = 0.f;
@@ -739,7 +744,7 @@ k_attn_finalize(const unsigned long long* __restrict__ mass, const int32_t* __re
         if (m & kMassNotFinite) {
           s = __int_as_float(0x7fc00000);
         } else {
-          s = __ll2float_rn(static_cast<long long>(m)) * (1.0f / static_cast<float>(1ull << kAttnMassFracBits));
+          s = __ll2float_rn(static_cast<long long>(m)) * unit;
           s = s / static_cast<float>(static_cast<int64_t>(Hq) * nq);
         }
       }
@@ -861,7 +866,8 @@ cudaError_t launch_attn_finalize(const avtp_layout_t& L, const avtp_score_args_t
                        static_cast<const int32_t*>(ws_at<int32_t>(ws, p.ktile_cu)),
                        static_cast<const int32_t*>(ws_at<int32_t>(ws, p.ktile_img)),
                        static_cast<const int4*>(ws_at<int4>(ws, p.tile_info)), sa.n_q_heads,
-                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.text_cu)), L.n_images, scores, img_sums,
+                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.text_cu)),
+                       static_cast<const int32_t*>(ws_at<int32_t>(ws, p.meta)), L.n_images, scores, img_sums,
                        static_cast<const DevStatus*>(ws_at<DevStatus>(ws, p.status)));
 }
 

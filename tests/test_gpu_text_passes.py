@@ -156,6 +156,22 @@ def test_scores_with_a_loose_text_bound(supplied):
         assert_scores_close(scores.cpu().numpy(), ref, lay.visual_mask())
 
 
+def test_mass_of_one_key_over_very_many_queries():
+    """Every row of a request puts all of its mass on one key: 2^23 rows, whose sum at 40 fraction
+    bits would reach the accumulator's top bit. The score is 1."""
+    Hq, d, n_text = 128, 64, 65536
+    L = avtp.Layout.from_host([0, 1 + n_text], [0, 1], [0], [1])
+    q = torch.zeros(1 + n_text, Hq, d, device="cuda", dtype=torch.bfloat16)
+    q[:, :, 0] = 1.0
+    k = torch.zeros(1 + n_text, 1, d, device="cuda", dtype=torch.bfloat16)
+    k[0, 0, 0] = 4.0
+    lse = torch.full((Hq, 1 + n_text), 4.0, device="cuda")  # the logit of the image's only token: probability 1
+    scores, sums = avtp.score(L, "text_attention", q=q, k=k, softmax_scale=1.0, lse=lse, path="tensor")
+    # lse2 and z2 are products of 4 with log2(e), each rounded once: within 2^-20 of each other
+    assert abs(float(scores[0]) - 1.0) < 4e-6
+    assert abs(int(sums[0]) - 2 ** 32) < 4e-6 * 2 ** 32
+
+
 @pytest.mark.parametrize("bad", [{"cu_seqlens": [0, 900, 200]}, {"cu_seqlens": [0, -5, 200]},
                                  {"cu_seqlens": [7, 100, 200]}, {"img_start": [0, 180]}, {"img_len": [60, 0]}])
 def test_last_token_logits_beside_a_refused_layout(bad):
