@@ -307,3 +307,15 @@ def test_binding_structs_match_the_c_layout(tmp_path):
         for f, _ in py._fields_:
             assert got[(c_name, f)] == getattr(py, f).offset, (c_name, f)
 
+
+def test_layout_counts_follow_its_host_arrays():
+    """A program that refills a layout for its next batch gets the next batch's counts."""
+    lay = avtp.Layout.from_host([0, 100, 180], [0, 2, 3], [5, 40, 1], [30, 20, 60], device="cpu")
+    assert lay.n_text == 70 and lay.n_vis_per_request.tolist() == [50, 60]
+    lay.host["img_len"][1] = 2
+    assert lay.n_text == 88 and lay.n_vis_per_request.tolist() == [32, 60]
+    lay.host["img_cu"][1] = 1
+    assert lay.n_text == 88 and lay.n_vis_per_request.tolist() == [30, 62]
+    lay.host = dict(cu_seqlens=np.array([0, 50, 60], dtype=np.int32), img_cu=np.array([0, 1, 1], dtype=np.int32),
+                    n_vis=np.array([40, 0], dtype=np.int32))
+    assert lay.n_text == 20 and lay.n_vis_per_request.tolist() == [40, 0]
