@@ -1089,7 +1089,7 @@ def run_timeline(args):
 # ---------------------------------------------------------------- forward timeline (diagnostic)
 def run_timeline_forward(args):
     """The attention forward in the timeline build (-DAVTP_TIMELINE): clock stamps per key
-    block of the CTA with the most key blocks (head 0), medians over its steady blocks and
+    block of the CTA of the last request's last query tile (head 0), medians over its steady blocks and
     over calls, in SM cycles: the block period, the softmax's phases and the MMA-issuing
     thread's. Not a bench line: the stamps add stores to the kernel."""
     os.environ["AVTP_TIMELINE"] = "1"

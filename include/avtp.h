@@ -227,7 +227,7 @@ AVTP_API avtp_status_t avtp_attn_forward(const avtp_layout_t* layout, const avtp
                                          void* workspace, size_t workspace_bytes, avtp_stream_t stream);
 
 /* Diagnostic: per-key-block clock stamps (SM cycles) of the last avtp_attn_forward call's
- * first CTA, the query tile with the most key blocks, head 0, for its first max_blocks (at
+ * first CTA, the last query tile of the last request, head 0, for its first max_blocks (at
  * most 256; the rest of out is left untouched) key blocks. Available in the library's
  * timeline build (compiled with AVTP_TIMELINE); the default build returns
  * AVTP_ERR_UNSUPPORTED. out: host int64 [max_blocks][10]: per block j, from softmax warp 0

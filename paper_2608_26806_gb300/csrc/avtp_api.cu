@@ -284,7 +284,7 @@ static avtp_status_t forward_args(const avtp_layout_t* L, const avtp_score_args_
   if (f->v_stride < Hkv * d || f->o_stride < Hq * d) return AVTP_ERR_INVALID_ARG;
   if (f->v_stride % 8 != 0 || f->o_stride % 4 != 0) return AVTP_ERR_UNSUPPORTED;
   if (!aligned16(f->v) || !aligned16(f->o)) return AVTP_ERR_UNSUPPORTED;
-  // query tiles x heads, the forward's grid: (T / 128 + R) * Hq CTAs
+  // query tiles x heads, at least as many as the forward's units: a counter of 32 bits deals them
   if ((L->n_tokens / 128 + L->n_requests) * Hq > 0x7fffffffLL) return AVTP_ERR_RANGE;
   *sa_out = sa;
   return AVTP_OK;

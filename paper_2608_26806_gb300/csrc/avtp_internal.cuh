@@ -63,7 +63,7 @@ struct DevStatus {
   int32_t code;
   int32_t layout_ok;
   int32_t detail;  // index of the first offending item, for debugging
-  uint32_t pool;   // tokens the criterion-A scoring kernel's warps have drawn from its pool
+  uint32_t pool;   // drawn so far: tokens by the criterion-A scoring's warps, or units by the forward's CTAs
 };
 
 __device__ __forceinline__ void record_error(DevStatus* st, int32_t code, int32_t detail) {

@@ -37,8 +37,8 @@
 // costs no precision in either (against 64 bits: O and the LSE are as far off as with a
 // maximum of every block).
 //
-// The kernel is persistent, a CTA per SM, units taken from a counter, those with the most key
-// blocks first: the next unit's queries and first keys arrive while the last block of the
+// The kernel is persistent, a CTA per SM, units taken from a counter in the packed order from
+// its end, so that within a request those with the most key blocks come first: the next unit's queries and first keys arrive while the last block of the
 // one before is under way, and its S runs during the rows' way out. Against a CTA per unit:
 // 206 -> 196 us the call over 5960 tokens (28 heads), 1104 -> 1028 us over eight requests of
 // 34423 tokens.
@@ -140,7 +140,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // Diagnostic timeline build (-DAVTP_TIMELINE): clock stamps of slot 0 of the grid's first CTA
-// (a tile with the most key blocks), per key block j. Stamps: 0-4 from softmax warp 0
+// (the last request's last tile), per key block j. Stamps: 0-4 from softmax warp 0
 // (loop top, S ready, P of the first half computed, of the second half, P handed over); 5-9
 // from the MMA thread (S_j: entry, issued; P_j V_j: entry, operands ready, issued). Read with
 // avtp_forward_timeline().
@@ -294,7 +294,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
         if (more) {
           const int tu = static_cast<int>(u / n_sub);
           un.x = static_cast<int>(u - static_cast<int64_t>(tu) * n_sub);
-          const int tq = n_rows - 1 - tu;  // a request's tiles with the most key blocks first
+          const int tq = n_rows - 1 - tu;  // the last request's tiles first, each request's from its end
           const int r = upper_index(pre, a.R, tq);
           un.cu = near ? sy.start[r] : a.cu[r];
           un.end = near ? sy.end[r] : a.cu[r + 1];
@@ -333,8 +333,8 @@ k_attn_fwd(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUt
           break;
         }
         // taken when the unit's last blocks are under way and not before, so that the CTA that
-        // is through first takes the heaviest unit left (252 units of 1 to 17 blocks on 152 SMs:
-        // 48 us when each CTA took its second unit with its first, 42 us so)
+        // is through first takes the next unit, in one request the heaviest left (252 units of 1
+        // to 17 blocks on 152 SMs: 48 us when each CTA took its second unit with its first, 42 us so)
         u = total;
         if (total > gridDim.x) {
           pdl_wait();  // the validation kernel resets the counter

@@ -52,8 +52,9 @@ __device__ T block_exclusive_scan(int n, F value, T* out, T* s_warp) {
 }
 
 // Layout arrays are staged in shared memory when they fit. Kept small (10 KiB) so
-// that this one-CTA kernel can share an SM with a CTA of the scoring kernel,
-// which is launched while this kernel still runs.
+// that this one-CTA kernel can share an SM with a CTA of the hidden-variation scoring,
+// which is launched while this kernel still runs. (With the text-query bookkeeping the
+// lists below take 8 KiB more; the scoring kernels behind that wait for this one.)
 constexpr int kStageInts = 2560;
 
 // Prefixes of the two passes' lists kept in shared memory for the search of the CTAs' runs.

@@ -147,9 +147,9 @@ __device__ void block_scan_inplace(int32_t* a, int n, int32_t* s_warp) {
   __syncthreads();
 }
 
-// 64 registers a thread: on large batches (no SMs left free) a CTA of the selection
-// kernel (256 threads, up to 128 registers) can then start on the same SM as this one
-// and wait there for the scores.
+// 64 registers a thread: half of the SM's stay free. Where no SMs are left to it, a CTA of
+// k_select (256 threads of 63 registers) can start on the same SM as this one and wait there
+// for the scores; one of k_alloc_select (184 registers) cannot.
 __global__ void __maxnreg__(64)
 k_score_hvar(const __nv_bfloat16* __restrict__ h_cur, int64_t cur_stride, const __nv_bfloat16* __restrict__ h_prior,
              int64_t prior_stride, int D, const int32_t* __restrict__ cu, int R, const int32_t* __restrict__ icu,

@@ -249,15 +249,18 @@ def test_host_validation_of_forward_arguments(lib):
     assert _forward(lib, lay, _attn_args(), _fwd_args(), ws=FAKE + 16) == avtp.ERR_WORKSPACE
 
 
-def test_forward_workspace_holds_the_transposed_values(lib):
-    lay = _layout(n_req=2, n_img=5, T=10000)
+@pytest.mark.parametrize("n_req", [2, 63, 64, 1000])
+def test_forward_workspace_adds_the_unit_prefix(lib, n_req):
+    """Beyond the scoring with a supplied LSE the forward keeps one prefix over the requests."""
+    lay = _layout(n_req=n_req, n_img=5, T=10000)
     a, b = ctypes.c_size_t(), ctypes.c_size_t()
-    sa = _attn_args()
-    assert lib.avtp_workspace_size(ctypes.byref(lay), ctypes.byref(sa), ctypes.byref(a)) == avtp.OK
+    sa, supplied = _attn_args(), _attn_args()
+    supplied.lse, supplied.lse_stride = FAKE, 10000
+    assert lib.avtp_workspace_size(ctypes.byref(lay), ctypes.byref(supplied), ctypes.byref(a)) == avtp.OK
     fa = _fwd_args(T=10000)
     assert lib.avtp_forward_workspace_size(ctypes.byref(lay), ctypes.byref(sa), ctypes.byref(fa),
                                            ctypes.byref(b)) == avtp.OK
-    assert b.value >= 8 * 128 * 10000 * 2 and b.value % 256 == 0
+    assert b.value == a.value + (4 * (n_req + 1) + 255) // 256 * 256
 
 
 def test_forward_timeline_needs_the_timeline_build(lib):
