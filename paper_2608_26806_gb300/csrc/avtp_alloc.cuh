@@ -173,9 +173,10 @@ __device__ __forceinline__ float u128_to_float(u128 v) {
 // would get more than one token. The general stage it stands in for keeps remainders of
 // three words in shared memory and ranks every image against every other: with it the rule
 // and the selection of four requests of 64 images took 127 us in one kernel, with this 41.
-// Four images a lane up to 128 and eight beyond: a request of 129 images of 64 tokens, the whole
-// stage, 211 -> 40 us, of 256 552 -> 90 (of 65 tokens, hidden 3584, 43 and 92). The two are apart so that the smaller carries no more
-// code (which is fetched cold) and registers than it needs; eight take 244 registers.
+// Four images a lane up to 128 and eight beyond: a request of 129 images of 64 tokens, the
+// whole stage, 211 -> 40 us, of 256 552 -> 90 (of 65 tokens, hidden 3584, 43 and 92). The two
+// are apart so that the smaller carries no more code (which is fetched cold) and registers than
+// it needs; eight take 244 registers.
 constexpr int kMultiImages = 256;
 
 template <bool kRel, int kMultiLanes>

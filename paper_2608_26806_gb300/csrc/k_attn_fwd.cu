@@ -38,10 +38,10 @@
 // maximum of every block).
 //
 // The kernel is persistent, a CTA per SM, units taken from a counter in the packed order from
-// its end, so that within a request those with the most key blocks come first: the next unit's queries and first keys arrive while the last block of the
-// one before is under way, and its S runs during the rows' way out. Against a CTA per unit:
-// 206 -> 196 us the call over 5960 tokens (28 heads), 1104 -> 1028 us over eight requests of
-// 34423 tokens.
+// its end, so that within a request those with the most key blocks come first: the next unit's
+// queries and first keys arrive while the last block of the one before is under way, and its S
+// runs during the rows' way out. Against a CTA per unit: 206 -> 196 us the call over 5960
+// tokens (28 heads), 1104 -> 1028 us over eight requests of 34423 tokens.
 //
 // Measured (32 query heads, 8 KV heads, d = 128, one request of 10368 tokens, this kernel
 // alone): 480 us at the full clock, 1830 TFLOP/s; up to 580 us where the power limit lowers
